@@ -306,13 +306,10 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
     P.sigma_s = ss;
     P.q = q;
     P.inflow = inflow;
-    int dev = 0, clk_khz = 0;
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&clk_khz, cudaDevAttrClockRate, dev));
-    if (clk_khz <= 0) clk_khz = 2000000;
-    P.wait_cycles = (long long)(opt->wait_limit_s * clk_khz * 1000.0);
-    P.num_sms = device_sm_count();
-    if (P.num_sms <= 0) return fail(GSIS_ERR_CUDA, "cannot query the device");
+    const DeviceInfo di = device_info();
+    if (di.sms <= 0) return fail(GSIS_ERR_CUDA, "cannot query the device");
+    P.wait_cycles = (long long)(opt->wait_limit_s * di.clock_khz * 1000.0);
+    P.num_sms = di.sms;
     CK(prepare_kernels(std::max(P.K, 1), P.fp32, P.pt));
     if (P.K > 0) {
         const int per_sm = std::max(1, sweep_max_active_blocks(P.fp32, P.pt));
@@ -416,6 +413,7 @@ gsis_options sweep_options(const gsis_options* o)
     r.cfl_p = 0.0;
     r.beta = 0.0;
     r.spatial_order = 1;
+    r.scheme = GSIS_SCHEME_SI;   // no synthetic solve follows: its operator and hierarchy are not built
     return r;
 }
 

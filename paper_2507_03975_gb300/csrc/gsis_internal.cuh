@@ -260,7 +260,11 @@ bool strip_batch_rec(const Plan& P, int cl, void* out, size_t* bytes);
 bool prepare_strip_batch(int cl, size_t bytes);
 cudaError_t launch_strip_batch(const void* tab, int n, int cl, size_t bytes, cudaStream_t st);
 
-int device_sm_count();
+// The current device's SM count and peak SM clock (sms = 0: no device).
+struct DeviceInfo {
+    int sms, clock_khz;
+};
+DeviceInfo device_info();
 void set_last_error(int code, const char* msg);   // message returned by gsis_last_error()
 
 // ------------------------------------------------------------ device helpers

@@ -22,6 +22,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
+#include <climits>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -64,13 +66,17 @@ __global__ void coef_kernel(int nx, int ny, int K, const double* __restrict__ dx
 // (Eqs. (elem_mtx_M), (Gamma_ij_com2) on the Cartesian mesh:
 // Gamma = 2 / (3 (sigma_i h_i + sigma_j h_j)); boundary
 // beta = 2/(3 sigma_i h_i) + 1/4 from Eq. (macro_bc_delta_flux)), input checks
-// (opacities, sources and inflow finite; opacities non-negative).
+// (opacities, sources and inflow finite; opacities non-negative).  Bound by
+// the FP64 pipe: thirteen divisions a cell.  synth = 0 (a kinetic step alone,
+// source iteration): no synthetic operator and no HoT weights, and with no
+// pseudo-time and no intensity gradient no division is left (256x256:
+// 26.7 -> 4.5 us).
 __global__ void cell_setup_kernel(int nx, int ny, const double* __restrict__ dx,
                                   const double* __restrict__ dy, const double* __restrict__ sa,
                                   const double* __restrict__ ss, const double* __restrict__ q,
                                   const double* __restrict__ inflow, int n_inflow,
                                   double shift0, double cfl_p, double beta, double* sigt, float* sigt_f,
-                                  double* shift, float* shift_f, double* diag, double* cx,
+                                  double* shift, float* shift_f, int synth, double* diag, double* cx,
                                   double* cy, double* hw, double* bface, double* gw, float* gw_f,
                                   float* sigt_d, int* err)
 {
@@ -89,25 +95,26 @@ __global__ void cell_setup_kernel(int nx, int ny, const double* __restrict__ dx,
         // neighbour optical distances |sigma_i r^L - sigma_j r^R|
         double th = 0.0;
         double gE = 0.0, gW = 0.0, gN = 0.0, gS = 0.0;
-        if (i + 1 < nx) {
+        const bool dist = synth || beta > 0.0;
+        if (dist && i + 1 < nx) {
             const double o = 0.5 * (st * hx + (sa[c + 1] + ss[c + 1]) * dx[i + 1]);
             th = fmax(th, o);
-            gE = 1.0 / (3.0 * o);
+            if (synth) gE = 1.0 / (3.0 * o);
         }
-        if (i > 0) {
+        if (dist && i > 0) {
             const double o = 0.5 * (st * hx + (sa[c - 1] + ss[c - 1]) * dx[i - 1]);
             th = fmax(th, o);
-            gW = 1.0 / (3.0 * o);
+            if (synth) gW = 1.0 / (3.0 * o);
         }
-        if (j + 1 < ny) {
+        if (dist && j + 1 < ny) {
             const double o = 0.5 * (st * hy + (sa[c + nx] + ss[c + nx]) * dy[j + 1]);
             th = fmax(th, o);
-            gN = 1.0 / (3.0 * o);
+            if (synth) gN = 1.0 / (3.0 * o);
         }
-        if (j > 0) {
+        if (dist && j > 0) {
             const double o = 0.5 * (st * hy + (sa[c - nx] + ss[c - nx]) * dy[j - 1]);
             th = fmax(th, o);
-            gS = 1.0 / (3.0 * o);
+            if (synth) gS = 1.0 / (3.0 * o);
         }
         const double ref = fmin(hx, hy);
         double sh = shift0;   // 1/(c dt) of a time step (0 when steady)
@@ -116,6 +123,7 @@ __global__ void cell_setup_kernel(int nx, int ny, const double* __restrict__ dx,
         shift[c] = sh;
         if (shift_f) shift_f[c] = (float)sh;
         if (sigt_d) sigt_d[c] = (float)(st + sh);
+        if (!synth && !gw) continue;
         // D = V sigma_a + sum_int A Gamma + sum_bnd A beta
         double d = hx * hy * a + hy * (gE + gW) + hx * (gN + gS);
         const double bx = 2.0 / (3.0 * st * hx) + 0.25, by = 2.0 / (3.0 * st * hy) + 0.25;
@@ -1237,12 +1245,26 @@ int sweep_fp64_occupancy()
 
 }  // namespace
 
-int device_sm_count()
+// Asked of the driver once per device: both are constants of the device, and
+// the clock rate costs 0.3-0.6 ms a query (64x64 S8 transport sweep: 684 us a
+// call with two queries, 120-205 us without them and the set-up below).
+DeviceInfo device_info()
 {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    return n;
+    constexpr int kMaxDev = 64;
+    static std::atomic<long long> known[kMaxDev];   // sms << 32 | clock_khz; 0: not asked yet
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return DeviceInfo{0, 0};
+    long long v = dev < kMaxDev ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (v == 0) {
+        int n = 0, khz = 0;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess)
+            return DeviceInfo{0, 0};
+        if (khz <= 0) khz = 2000000;
+        v = ((long long)n << 32) | (long long)khz;
+        if (dev < kMaxDev) known[dev].store(v, std::memory_order_relaxed);
+    }
+    return DeviceInfo{(int)(v >> 32), (int)(v & 0xffffffffll)};
 }
 
 cudaError_t launch_setup(const Plan& P, cudaStream_t st)
@@ -1260,7 +1282,8 @@ cudaError_t launch_cell_setup(const Plan& P, double cfl_p, double beta, cudaStre
 {
     cell_setup_kernel<<<grid_for(P.N, 256, P.num_sms * 8), 256, 0, st>>>(
         P.nx, P.ny, P.dx, P.dy, P.sigma_a, P.sigma_s, P.q, P.inflow, P.nbf * P.K, P.shift0, cfl_p, beta, P.sigt,
-        P.fp32 ? P.sigt_f : nullptr, P.shift, P.fp32 ? P.shift_f : nullptr, P.diag, P.cx, P.cy, P.hw,
+        P.fp32 ? P.sigt_f : nullptr, P.shift, P.fp32 ? P.shift_f : nullptr,
+        P.scheme == GSIS_SCHEME_GSIS || P.K == 0, P.diag, P.cx, P.cy, P.hw,
         P.bface, P.gw, P.gw_f, P.sigt_d, &P.status->error);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

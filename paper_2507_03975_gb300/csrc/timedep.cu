@@ -401,7 +401,8 @@ int td_start(Plan& P, const gsis_time_params* tp, int gsis, const double* rho0, 
 {
     const int g = grid_for(P.N, kRedBlock, P.num_sms * 8);
     const TdArgs a = td_args(P, tp, gsis);
-    CK(cudaMemcpyAsync(P.td.diag0, P.diag, (size_t)P.N * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    if (gsis)   // source iteration has no synthetic operator
+        CK(cudaMemcpyAsync(P.td.diag0, P.diag, (size_t)P.N * sizeof(double), cudaMemcpyDeviceToDevice, st));
     TIMED(GSIS_KCLASS_SETUP, 2, launch_td_init(P, a, g, rho0, T0, st));
     return GSIS_OK;
 }
