@@ -123,8 +123,9 @@ size_t layout(const Sizes& z, char* base, Plan* P)
     p.qmu = qbuf; p.qeta = qbuf ? qbuf + K : nullptr; p.qw = qbuf ? qbuf + 2 * K : nullptr;
     p.omu = qbuf ? qbuf + 3 * K : nullptr; p.oeta = qbuf ? qbuf + 4 * K : nullptr;
     p.ow = qbuf ? qbuf + 5 * K : nullptr;
-    int* ibuf = reinterpret_cast<int*>(take(3 * K * sizeof(int)));
+    int* ibuf = reinterpret_cast<int*>(take(5 * K * sizeof(int)));
     p.perm = ibuf; p.sidx = ibuf ? ibuf + K : nullptr; p.mpair = ibuf ? ibuf + 2 * K : nullptr;
+    p.rrep = ibuf ? ibuf + 3 * K : nullptr; p.rnext = ibuf ? ibuf + 4 * K : nullptr;
     p.dx = reinterpret_cast<double*>(take(z.nx * sizeof(double)));
     p.dy = reinterpret_cast<double*>(take(z.ny * sizeof(double)));
     p.acoef = reinterpret_cast<double*>(take(K * z.nx * sizeof(double)));
@@ -332,7 +333,7 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
                 if (kq == qd) perm.push_back(k);
             }
         std::vector<double> hq(6 * (size_t)K);
-        std::vector<int> hi(3 * (size_t)K, -1);
+        std::vector<int> hi(5 * (size_t)K, -1);
         for (int s = 0; s < K; ++s) {
             hq[s] = quad->mu[perm[s]];
             hq[K + s] = quad->eta[perm[s]];
@@ -363,6 +364,17 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
                 hi[2 * K + 2 * np] = k;
                 hi[2 * K + 2 * np + 1] = m;
                 ++np;
+            }
+        }
+        // directions of equal |mu|, |eta| (they share 1/d at a cell): first ones and chains
+        P.nrep = 0;
+        for (int s = 0; s < K; ++s) {
+            int f = 0;
+            while (std::fabs(hq[f]) != std::fabs(hq[s]) || std::fabs(hq[K + f]) != std::fabs(hq[K + s])) ++f;
+            if (f == s) hi[3 * K + P.nrep++] = s;
+            else {
+                while (hi[4 * K + f] >= 0) f = hi[4 * K + f];
+                hi[4 * K + f] = s;
             }
         }
         CK(cudaMemcpyAsync(const_cast<double*>(P.qmu), hq.data(), hq.size() * sizeof(double),

@@ -96,6 +96,8 @@ struct Plan {
     const int* perm;                // s -> original k
     const int* sidx;                // original k -> s
     const int* mpair;               // [K/2][2] original k of the x-reflection pairs (mu, eta), (-mu, eta), equal w
+    const int* rrep; const int* rnext;   // [nrep] first directions of equal |mu|, |eta|; [K] the next such, or -1
+    int nrep;
     int has_mpair;                  // the quadrature has such pairs: moments take the paired sums
     // per-direction coefficients |mu_s|/dx_i [K][nx], |eta_s|/dy_j [K][ny]
     const double* acoef; const double* bcoef;
