@@ -18,6 +18,7 @@
 #include "gsis.h"
 #include "gsis_internal.cuh"
 #include "host.h"
+#include "moments_fixed.cuh"
 
 using namespace gsis;
 
@@ -126,6 +127,7 @@ size_t layout(const Sizes& z, char* base, Plan* P)
     int* ibuf = reinterpret_cast<int*>(take(5 * K * sizeof(int)));
     p.perm = ibuf; p.sidx = ibuf ? ibuf + K : nullptr; p.mpair = ibuf ? ibuf + 2 * K : nullptr;
     p.rrep = ibuf ? ibuf + 3 * K : nullptr; p.rnext = ibuf ? ibuf + 4 * K : nullptr;
+    p.mquad = z.fp32 ? nullptr : reinterpret_cast<MomQuad*>(take((K + 3) / 4 * sizeof(MomQuad)));
     p.dx = reinterpret_cast<double*>(take(z.nx * sizeof(double)));
     p.dy = reinterpret_cast<double*>(take(z.ny * sizeof(double)));
     p.acoef = reinterpret_cast<double*>(take(K * z.nx * sizeof(double)));
@@ -377,6 +379,33 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
                 hi[4 * K + f] = s;
             }
         }
+        // reflection quads (mu, eta), (-mu, eta), (mu, -eta), (-mu, -eta) of one
+        // weight: the FP64 moments then sum in fixed point (moments_fixed.cuh)
+        std::vector<MomQuad> quads;
+        P.has_mquad = !P.fp32 && K % 4 == 0;
+        for (int s = 0; s < K && P.has_mquad; ++s) {
+            const double m = hq[s], e = hq[K + s], w = hq[2 * K + s];
+            if (!(m != 0.0) || !(e != 0.0) || !(w < 2.0)) P.has_mquad = 0;
+            if (!(m > 0.0 && e > 0.0)) continue;
+            MomQuad q{};
+            for (int r = 0; r < 4; ++r) {
+                int t = 0;   // quads take distinct directions: a repeated direction is not a quad's
+                while (t < K && !(hq[t] == (r & 1 ? -m : m) && hq[K + t] == (r & 2 ? -e : e) && hq[2 * K + t] == w)) ++t;
+                q.s[r] = t;
+                if (t == K || (r == 0 && t != s)) P.has_mquad = 0;
+            }
+            const double cf[6] = {w, w * m, w * e, w * m * m, w * m * e, w * e * e};
+            for (int t = 0; t < 6; ++t) {
+                const unsigned long long c = (unsigned long long)std::nearbyint(std::ldexp(cf[t], 62));
+                q.c[t][0] = (unsigned)(c >> 32);
+                q.c[t][1] = (unsigned)c;
+            }
+            quads.push_back(q);
+        }
+        if (quads.size() * 4 != (size_t)K) P.has_mquad = 0;
+        if (P.has_mquad)
+            CK(cudaMemcpyAsync(const_cast<MomQuad*>(P.mquad), quads.data(), quads.size() * sizeof(MomQuad),
+                               cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(const_cast<double*>(P.qmu), hq.data(), hq.size() * sizeof(double),
                            cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(const_cast<int*>(P.perm), hi.data(), hi.size() * sizeof(int),

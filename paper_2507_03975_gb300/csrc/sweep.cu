@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "gsis_internal.cuh"
+#include "moments_fixed.cuh"
 
 namespace gsis {
 
@@ -834,7 +835,67 @@ struct MomArgs {
     const double* rho_new;                                  // GSIS correction of P (or null)
     const int* done;
     const int* pairs;   // [K/2][2] x-reflection pairs (original k, the first with mu > 0), or null
+    const MomQuad* quads;   // [K/4] reflection quads (FP64), or null
 };
+
+// FP64 moments of one cell by plain multiply-adds in the original direction
+// order (cells that the fixed-point sums do not cover).
+template <bool WITH_F, bool WITH_P>
+__device__ __forceinline__ void moments_plain_cell(const MomArgs<double>& a, int c, double* out)
+{
+    double r = 0.0, fx = 0.0, fy = 0.0, pxx = 0.0, pxy = 0.0, pyy = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < a.K; ++k) {
+        const double v = a.I[(size_t)a.sidx[k] * a.N + c], w = a.w[k], m = a.mu[k], e = a.eta[k];
+        r = fma(w, v, r);
+        if (WITH_F) {
+            fx = fma(w * m, v, fx);
+            fy = fma(w * e, v, fy);
+        }
+        if (WITH_P) {
+            pxx = fma(w * m * m, v, pxx);
+            pxy = fma(w * m * e, v, pxy);
+            pyy = fma(w * e * e, v, pyy);
+        }
+    }
+    out[0] = r;
+    if (WITH_F) { out[1] = fx; out[2] = fy; }
+    if (WITH_P) { out[3] = pxx; out[4] = pxy; out[5] = pyy; }
+}
+
+// FP64 moments over reflection quads in fixed point (moments_fixed.cuh),
+// one thread per cell.
+template <bool WITH_F, bool WITH_P>
+__device__ __forceinline__ void moments_quad_body(const MomArgs<double>& a, int bid, int nblk)
+{
+    constexpr int NM = WITH_P ? 6 : WITH_F ? 3 : 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    MomQuad* tab = reinterpret_cast<MomQuad*>(smem_raw);
+    const int nq = a.K / 4;
+    for (int t = threadIdx.x; t < nq * 16; t += blockDim.x) {
+        unsigned v = reinterpret_cast<const unsigned*>(a.quads)[t];
+        if ((t & 15) >= 4 && (t & 1)) v >>= 32 - FixedMoments<NM>::kFrac;
+        reinterpret_cast<unsigned*>(tab)[t] = v;
+    }
+    __syncthreads();
+    for (int c = bid * blockDim.x + threadIdx.x; c < a.N; c += nblk * blockDim.x) {
+        FixedMoments<NM> f;
+        double o[6];
+        if (!f.run(tab, nq, a.I, (size_t)a.N, c, o)) moments_plain_cell<WITH_F, WITH_P>(a, c, o);
+        if (a.rho) a.rho[c] = o[0];
+        if (WITH_F) {
+            a.Fx[c] = o[1];
+            a.Fy[c] = o[2];
+        }
+        if (WITH_P) {
+            double d = 0.0;   // moments of I + (rho_new - rho_half)/4pi: + drho/3 on the diagonal
+            if (a.rho_new) d = (a.rho_new[c] - o[0]) / 3.0;
+            a.Pxx[c] = o[3] + d;
+            a.Pxy[c] = o[4];
+            a.Pyy[c] = o[5] + d;
+        }
+    }
+}
 
 // Per cell, in original direction order k = 0..K-1:
 // rho = sum w I, F = sum w Omega I, P = sum w Omega Omega I.
@@ -845,11 +906,17 @@ __device__ __forceinline__ void moments_body(const MomArgs<T>& a, int bid, int n
     T* cf = reinterpret_cast<T*>(smem_raw);                     // [K][6]
     int* sk = reinterpret_cast<int*>(cf + 6 * a.K);             // [K]
     if (a.done && ld_volatile_int(a.done)) return;
+    if constexpr (sizeof(T) == 8) {
+        if (a.quads) {
+            moments_quad_body<WITH_F, WITH_P>(a, bid, nblk);
+            return;
+        }
+    }
     if (!WITH_P && a.pairs) {
         // Directions in x-reflection pairs k1 = (mu, eta), k2 = (-mu, eta)
         // with one weight: rho += w (I1 + I2), F_x += w mu (I1 - I2),
-        // F_y += w eta (I1 + I2): five FP64 operations per pair instead of
-        // six (the FP64 pipe bounds this kernel).
+        // F_y += w eta (I1 + I2): five operations per pair instead of six
+        // (FP32, and FP64 sets without reflection quads).
         const int np = a.K / 2;
         T* cp = cf;                                             // [np][3]: w, w mu, w eta of k1
         int* sp = reinterpret_cast<int*>(cf + 3 * np);          // [np][2]: sorted indices of k1, k2
@@ -1113,6 +1180,20 @@ cudaError_t launch_sweep_batch_t(const BatchTables& bt, cudaStream_t st)
     return cudaGetLastError();
 }
 
+// The fixed-point sums, except in the second-order scheme: its limiter
+// amplifies a rounding difference of 1e-16 to 3e-10 within 250 iterations
+// (256^2 S12 channel), so its sums keep their order and their bits.
+const MomQuad* moments_quads(const Plan& P) { return P.has_mquad && P.order != 2 ? P.mquad : nullptr; }
+
+// Blocks of the cell moments: one cell per thread over reflection quads (no
+// nearly empty last turn: 1024^2 would take 3.4 turns of 8 blocks per SM),
+// else a grid-stride loop that re-uses the block's coefficient table.
+template <typename T>
+int moments_blocks(const Plan& P)
+{
+    return grid_for(P.N, kRedBlock, sizeof(T) == 8 && moments_quads(P) ? INT_MAX : P.num_sms * 8);
+}
+
 template <typename T>
 size_t moments_smem(int K)
 {
@@ -1142,6 +1223,7 @@ cudaError_t launch_moments_t(const Plan& P, bool with_F, bool with_P, double* rh
     a.I = static_cast<const T*>(P.I);
     a.sidx = P.sidx;
     a.pairs = P.has_mpair ? P.mpair : nullptr;
+    a.quads = moments_quads(P);
     a.mu = P.omu;
     a.eta = P.oeta;
     a.w = P.ow;
@@ -1152,7 +1234,7 @@ cudaError_t launch_moments_t(const Plan& P, bool with_F, bool with_P, double* rh
     a.rho_new = gsis_correct ? P.rho_m : nullptr;
     a.done = force ? nullptr : &P.status->done;
     const size_t smem = moments_smem<T>(P.K);
-    const int grid = grid_for(P.N, kRedBlock, P.num_sms * 8);
+    const int grid = moments_blocks<T>(P);
     if (P.order != 2) {   // cells and boundary faces in one launch
         static_assert(kRedBlock == 256, "the boundary-flux blocks take 256 threads");
         const BfArgs<T> f = bflux_args<T>(P, fb_out, a.done);
@@ -1473,13 +1555,14 @@ int mom_batch_rec_t(const Plan& P, bool with_F, void* out)
     r.m.I = static_cast<const T*>(P.I);
     r.m.sidx = P.sidx;
     r.m.pairs = P.has_mpair ? P.mpair : nullptr;
+    r.m.quads = moments_quads(P);
     r.m.mu = P.omu; r.m.eta = P.oeta; r.m.w = P.ow;
     r.m.rho = P.rho_h;
     r.m.Fx = with_F ? P.Fx : nullptr;
     r.m.Fy = with_F ? P.Fy : nullptr;
     r.m.done = &P.status->done;
     r.f = bflux_args<T>(P, P.fb, &P.status->done);
-    r.mblocks = grid_for(P.N, kRedBlock, P.num_sms * 8);
+    r.mblocks = moments_blocks<T>(P);
     std::memcpy(out, &r, sizeof(r));
     return r.mblocks + grid_for((long long)P.nbf * 32, kRedBlock, P.num_sms * 4);
 }
