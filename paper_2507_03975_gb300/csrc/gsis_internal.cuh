@@ -13,7 +13,6 @@ constexpr int kWarp = 32;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxK = 4096;            // directions per quadrature (host-side check)
 constexpr int kMaxSide = (1 << 20) - 1; // cells per mesh side
-constexpr int kSweepMaxPairs = 12;      // (compute, copy) warp pairs per sweep CTA, at most: as many as fit
 constexpr size_t kSweepSmemCap = 231424; // dynamic shared memory a sweep CTA may take (the 227 KB opt-in less 1 KB)
 constexpr int kRedBlock = 256;          // threads per reduction / stencil block
 constexpr int kMaxCgBlocks = 1024;      // partials capacity of the fixed-order grid reductions
@@ -306,6 +305,18 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* b, unsigned pa
 {
     unsigned ok;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(smem_addr(b)), "r"(parity)
+                 : "memory");
+    return ok != 0;
+}
+
+// The same without suspending the thread.
+__device__ __forceinline__ bool mbar_test(unsigned long long* b, unsigned parity)
+{
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
                  "selp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(ok)
                  : "r"(smem_addr(b)), "r"(parity)

@@ -11,9 +11,10 @@
 // previous result (a register).  Lane 0 takes its south value from the band
 // below (its last-row results, handed over value by value through a global
 // row whose slots read "unwritten" until stored) or from the inflow on the
-// first band.  Each compute warp is paired with a copy warp that stages the
-// cell data of the coming steps in shared memory and fetches the south
-// values, so the compute warp touches global memory only to store results.
+// first band.  Each compute warp is paired with helper warps that stage the
+// cell data of the coming steps in shared memory, fetch the south values and
+// write the results out, so the compute warp touches global memory only to
+// hand its last row on.
 // Every wait is bounded and reports kErrTimeout instead of hanging.
 //
 // All intensities of the last sweep stay in HBM as I[s][cell] (needed by the
@@ -27,6 +28,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "gsis_internal.cuh"
@@ -292,8 +294,20 @@ struct SweepBatch {
     long long wait_cycles;
 };
 
-__device__ __forceinline__ double rcp_t(double d) { return 1.0 / d; }
-__device__ __forceinline__ float rcp_t(float d) { return __frcp_rn(d); }
+// 1/d of an FP32 diagonal in [2^-100, 2^100], correctly rounded: one Newton
+// step r + r (1 - d r) with the residual exact by FMA, from an approximation
+// within 1 ulp (Markstein 1990, "Computation of elementary functions on the
+// IBM RISC System/6000"; compared with __frcp_rn for every float of the
+// range: equal).  Six instructions that overlap from cell to cell;
+// __frcp_rn with its range checks took 136 cycles a cell, one after the
+// other, and set the pace of the FP32 sweep (2179 cycles per 16-step chunk).
+constexpr unsigned kRcpLo = (127u - 100u) << 23, kRcpHi = (127u + 100u) << 23;
+__device__ __forceinline__ float rcp_newton(float d)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return __fmaf_rn(r, __fmaf_rn(-d, r, 1.0f), r);
+}
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem)
@@ -349,92 +363,151 @@ template <> struct Bits<float> {
     }
 };
 
-// Shared-memory plan of one (compute, copy) warp pair.  A chunk is SEG
-// consecutive steps (64-byte row segments).  Each of the NBUF chunk buffers
-// holds, for the lane's own row, the cell data of the SEG cells the lane
-// updates in the chunk (padded rows: conflict-free column access), the
-// column coefficients of the SEG + 31 columns the skewed lanes touch, the
-// 1/d table rows of the chunk (FP64) and the SEG south values of lane 0.
-template <typename T, int XW, bool PRE, bool WIDE = false>
+// What the load warp tells the other warps of its pair about a chunk (in the
+// chunk's buffer): the unit, where its results and its hand-off row go, and
+// the adjoint source's coefficients.
+template <typename T>
+struct alignas(16) SweepHdr {
+    int task;                  // launch unit, -1: no more units
+    int nchunks, nx, rows;     // rows of the band inside the mesh
+    T* out;                    // I at (band row 0, sweep column 0)
+    T* eo;                     // this band's hand-off row, by column
+    int* err;
+    int t0, dr, dc, put_edge;  // first step of the chunk; strides of `out`; a band above reads the last row
+    T* ei;                     // the band below's hand-off row, or null (band 0)
+    const double* in;          // band 0: inflow of sweep column c at in[c * in_step], or null (vacuum)
+    long long in_step;
+    T cw, cm, ce;              // adjoint source w (a - mu bx - eta by)
+};
+
+// Shared-memory plan of one pair's warps.  A chunk is SEG consecutive steps
+// (64-byte row segments).  Each of the NBUF chunk buffers holds, for the
+// lane's own row, the cell data of the SEG cells the lane updates in the
+// chunk (padded rows: conflict-free column access), the column coefficients
+// of the SEG + 31 columns the skewed lanes touch, the 1/d table rows of the
+// chunk (FP64), the SEG south values of lane 0, the unit's row coefficients
+// and wall values (first chunk) and the header.
+template <typename T, int MODE>
 struct SweepSmem {
+    static constexpr bool PRE = sizeof(T) == 8;               // 1/d from the table
+    static constexpr int XW = sweep_xw(MODE);
+    // a preparation warp forms what the compute warp can take ready-made: 1/d
+    // in FP32, the combined source of the pseudo-time and adjoint forms
+    static constexpr bool PREP = !PRE || MODE == kSrcPseudoTime || MODE == kSrcAdjoint;
+    static constexpr int WARPS = PREP ? 4 : 3;                // compute, load, south [, preparation]
     static constexpr int SEG = 64 / (int)sizeof(T);
-    static constexpr int NBUF = 3;
+    // Buffers per pair: deeper queues hide more of the copies' latency, but the
+    // shared memory comes out of the L1 that the 64-byte windows, shifted by
+    // one cell from row to row, find their shared sectors in (FP64 1024^2
+    // S16: 3 buffers 0.89 ms, 4 1.04 ms; FP32 512^2 S12: 3, 4, 5 buffers 125,
+    // 98, 109 us).
+    static constexpr int NBUF = PRE ? 3 : 4;
     static constexpr int RS = SEG + 1;
     static constexpr int AW = SEG + 32;
     static constexpr int NW = (PRE ? 1 : 2) + XW;              // src, [sigt], [shift,] [I^m or I^n]
     static constexpr int W_SRC = 0;                           // window slots
     static constexpr int W_SIGT = 1;                          // FP32 only (no 1/d table)
     static constexpr int W_SHIFT = PRE ? 1 : 2;               // two extra windows only
-    static constexpr int W_IOLD = (PRE ? 1 : 2) + (XW >= 2 ? 1 : 0);   // extra windows only
+    static constexpr int W_IOLD = PRE ? 2 : 3;
     static constexpr int WIN = 32 * RS;
     static constexpr size_t r16(size_t b) { return (b + 15) / 16 * 16; }
     static constexpr size_t off_r = r16(sizeof(T) * (size_t)NW * WIN);
     static constexpr size_t off_a = off_r + (PRE ? (size_t)SEG * 32 * sizeof(double) : 0);
     static constexpr size_t off_e = off_a + r16(sizeof(T) * (size_t)AW);
-    static constexpr size_t off_h = off_e + r16(sizeof(T) * (size_t)SEG);   // unit index of the chunk
-    static constexpr size_t buf_bytes = off_h + 16;
-    static constexpr size_t bar_bytes = 64;                   // full[NBUF], empty[NBUF]
-    static constexpr size_t pair_bytes = bar_bytes + NBUF * buf_bytes;
-    // pairs per CTA: 8 (two chains per SM sub-partition), or in the WIDE
-    // form as many as the shared memory holds up to kSweepMaxPairs (the
-    // batched sweep: 64 problems 0.69 -> 0.55 ms; with staged write-out,
-    // the FP64 sweep of a problem with many units, below)
+    static constexpr size_t off_c = off_e + r16(sizeof(T) * (size_t)SEG);
+    static constexpr size_t off_h = off_c + 2 * 32 * sizeof(T);
+    static constexpr size_t buf_bytes = off_h + r16(sizeof(SweepHdr<T>));
+    static constexpr size_t bar_bytes = 4 * 8 * (size_t)NBUF;   // full, ready, done, empty
+    static constexpr size_t off_buf = r16(bar_bytes);
+    static constexpr size_t pair_bytes = off_buf + NBUF * buf_bytes;
+    // pairs per CTA: 8 (two chains per SM sub-partition) where the shared
+    // memory holds them (FP64 1024^2 S16: 6, 7, 8 pairs 0.985, 0.918, 0.887
+    // ms; the FP64 pipe is saturated by six chains, 18.4 cycles an operation)
     static constexpr size_t kFit = kSweepSmemCap / pair_bytes;
-    static constexpr size_t kWant = WIDE ? (size_t)kSweepMaxPairs : (size_t)8;
+    static constexpr size_t kWant = 8;
     static constexpr int PAIRS = (int)(kFit < kWant ? kFit : kWant);
+    static constexpr int THREADS = PAIRS * WARPS * 32;
     static constexpr size_t bytes = PAIRS * pair_bytes;
     static_assert(PAIRS >= 4, "a sweep CTA needs at least one pair per sub-partition");
-    static_assert(2 * NBUF * 8 <= bar_bytes, "barrier space");
+    static_assert(NBUF >= 3, "the preparation warp writes a chunk out two chunks behind");
 };
 
-// One persistent CTA per SM runs PAIRS warp pairs; a pair's copy warp
-// chooses the units (direction s, band), u = band * K + s, and hands each to
-// its compute warp in the header of the unit's first chunk buffer.  When the
-// whole grid is resident (every CTA checks in within a few microseconds) the
-// units are placed statically: pair p of CTA c takes u = p G + c + i PAIRS G, so
-// each SM's first units come from different bands and run at different
-// times; every unit is owned by a running pair and waits only on u - K.
-// Otherwise (part of the grid held back by other work on the GPU) the pairs
-// take units from a counter in increasing order, so a unit only waits on one
-// that a running pair took earlier.  One atomic decision picks the mode for
-// every CTA; the launch's last warp to leave re-arms the counters.
+// One persistent CTA per SM runs PAIRS "pairs" of a compute warp and its two
+// or three helpers; a pair's load warp chooses the units (direction s, band),
+// u = band * K + s, and hands each on in the headers of its chunk buffers.
+// When the whole grid is resident (every CTA checks in within a few
+// microseconds) the units are placed statically: pair p of CTA c takes
+// u = p G + c + i PAIRS G, so each SM's first units come from different
+// bands and run at different times; every unit is owned by a running pair and
+// waits only on u - K.  Otherwise (part of the grid held back by other work
+// on the GPU) the pairs take units from a counter in increasing order, so a
+// unit only waits on one that a running pair took earlier.  One atomic
+// decision picks the mode for every CTA; the launch's last warp to leave
+// re-arms the counters.
 //
-// Copy warp: for each chunk, cp.async of the window data into a free buffer
-// (arrival on the buffer's "full" barrier when the copies land), then the
-// south values of lane 0: the inflow on band 0, else the upstream band's
-// last-row results, polled until written (bounded).  Compute warp: waits on
-// "full", runs the SEG steps from shared memory, writes each result straight
-// to I, and the last lane also to this band's hand-off row, then arrives on
-// "empty".  Every wait is bounded; on time-out kErrTimeout is raised and the
-// warp leaves after its copies in flight have landed.
-template <typename T, int MODE, bool PRE, bool BATCH, bool WIDE = false>
-__global__ void __launch_bounds__(SweepSmem<T, sweep_xw(MODE), PRE, BATCH || WIDE>::PAIRS * 64, 1)
+// The time of a sweep with few units is the wavefront's critical path:
+// nx + ny steps plus, per band, a chunk and a hand-off.  So the compute warp
+// does nothing but the steps; what it used to do beside them (waiting with 32
+// arrivals per barrier, writing results out, FP32 reciprocals, the wall's
+// conditionals) took as long again:
+//
+//   load warp     cp.async of the window data into a free buffer, header.
+//                 Without a preparation warp it also writes finished chunks
+//                 out before it refills their buffer.
+//   south warp    lane 0's south values of a chunk: the inflow on band 0, else
+//                 the upstream band's last-row results, polled until written
+//                 (in a warp of its own: between the load warp's copies a
+//                 poll came a round trip to L2 late at every chunk).
+//   preparation   (PREP) per chunk, in place: FP32 1/d, the pseudo-time or
+//   warp          adjoint source; then writes out the chunk two behind.
+//   compute warp  SEG steps from shared memory, each result into the slot of
+//                 the source it used, the last lane's also to the band's
+//                 hand-off row.  Slots outside the mesh are computed like
+//                 the others, from the nearest cell's data: no lane inside
+//                 the mesh reads their results (lane l + 1 at step t reads
+//                 lane l of step t - 1, the same column), the west value is
+//                 set to the wall's at the lane's first column, and nothing
+//                 of them is written out.
+//
+// Every wait is bounded; on time-out kErrTimeout is raised and the warp leaves
+// after its copies in flight have landed.
+//
+// Before / after (one launch, us): FP64 64^2 S8 31 / 26, 256^2 S12 108 / 94
+// (per-ordinate source) and 189 / 150 (increment form), 200^2 S8 35 / 28 and
+// 51 / 40 (adjoint form), 1024^2 S16 919 / 887; FP32 641x470 S6 254 / 96,
+// 512^2 S12 190 / 98, batch of 24 problems 158 / 128.  Bounds now: FP64 with
+// many units, the pipe (1024^2 S16: 14.2 M warp operations of 18.4 cycles on
+// 152 SMs, 0.83 ms); with few, the chain of a step (265 cycles: three FP64
+// operations and a 64-bit shuffle); FP32, instruction issue of the four warps
+// of a pair and the load warp's 34 copy instructions a chunk.
+template <typename T, int MODE, bool BATCH>
+__global__ void __launch_bounds__(SweepSmem<T, MODE>::THREADS, 1)
 sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
 {
     constexpr bool PT = MODE == kSrcPseudoTime, ADJ = MODE == kSrcAdjoint, DELTA = MODE == kSrcDelta;
-    // FP32 and the WIDE form: results collected in shared memory and written
-    // out per chunk in coarser stores (fewer store instructions per step:
-    // one 8-byte store per step touches 32 rows); the FP64 latency-bound
-    // form writes each result at once (there the write-out would sit on the
-    // band hand-off path: 256^2 S12 channel 0.127 -> 0.141 ms when staged)
-    constexpr bool STAGE = sizeof(T) == 4 || WIDE;
-    using SM = SweepSmem<T, sweep_xw(MODE), PRE, BATCH || WIDE>;
+    using SM = SweepSmem<T, MODE>;
     using B = Bits<T>;
+    using Hdr = SweepHdr<T>;
+    constexpr bool PRE = SM::PRE, PREP = SM::PREP;
     constexpr int SEG = SM::SEG, NBUF = SM::NBUF, RS = SM::RS, NW = SM::NW;
+    constexpr int RPI = 32 / SEG;   // rows per copy or write-out instruction
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool copier = warp >= SM::PAIRS;
-    const int pair = copier ? warp - SM::PAIRS : warp;
+    const int role = warp / SM::PAIRS, pair = warp - role * SM::PAIRS;   // 0 compute, 1 load, 2 south, 3 preparation
     unsigned char* pbase = smem_raw + (size_t)pair * SM::pair_bytes;
-    unsigned long long* full = reinterpret_cast<unsigned long long*>(pbase);
-    unsigned long long* empty = full + NBUF;
-    auto buf = [&](int b) { return pbase + SM::bar_bytes + (size_t)b * SM::buf_bytes; };
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(pbase);   // data and header
+    unsigned long long* ready = full + NBUF;     // south values [, prepared]
+    unsigned long long* done_b = ready + NBUF;   // steps finished
+    unsigned long long* empty = done_b + NBUF;   // PREP: written out
+    auto buf = [&](int b) { return pbase + SM::off_buf + (size_t)b * SM::buf_bytes; };
 
     if (threadIdx.x < SM::PAIRS) {
         unsigned long long* f = reinterpret_cast<unsigned long long*>(smem_raw + (size_t)threadIdx.x * SM::pair_bytes);
         for (int b = 0; b < NBUF; ++b) {
-            mbar_init(f + b, 64);            // 32 cp.async arrivals + 32 lane arrivals
-            mbar_init(f + NBUF + b, 32);     // 32 compute lanes
+            mbar_init(f + b, 33);                        // 32 cp.async arrivals, the header
+            mbar_init(f + NBUF + b, PREP ? 2 : 1);       // south values [, preparation]
+            mbar_init(f + 2 * NBUF + b, 1);
+            mbar_init(f + 3 * NBUF + b, 1);
         }
     }
     __syncthreads();
@@ -446,10 +519,12 @@ sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
     unsigned* const c_exits = BATCH ? bt.exits : a1.exits;
     unsigned* const c_arrived = BATCH ? bt.arrived : a1.arrived;
     int* const c_mode = BATCH ? bt.mode : a1.mode;
+    int* const c_err = BATCH ? bt.err : a1.err;
 
-    __shared__ int cta_mode;
+    __shared__ int cta_mode, cta_stop;
     if (threadIdx.x == 0) {
         atomicAdd(c_arrived, 1u);
+        cta_stop = BATCH ? 0 : ld_volatile_int(a1.done) | ld_volatile_int(a1.err);
         const long long t0 = clock64();
         int m = 0;
         for (;;) {
@@ -463,18 +538,60 @@ sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
     __syncthreads();
     const bool placed = cta_mode == 1 && !(BATCH && bt.dynamic);
 
-    unsigned g = 0;   // chunks this pair has handled (buffer = g % NBUF)
-    int next_static = pair * G + (int)blockIdx.x;
-    bool first = true;
-    auto body = [&]() {
-    if (!BATCH) {
-        int stop = 0;
-        if (lane == 0) stop = ld_volatile_int(a1.done) | ld_volatile_int(a1.err);
-        if (__shfl_sync(kFull, stop, 0)) return;
-    }
-    for (;;) {
-        int task, prob = 0, ltask;   // launch unit, its problem and the unit within the problem
-        if (copier) {
+    // All lanes wait for the phase of chunk g; false (in all of them) on time-out.
+    auto wait_all = [&](unsigned long long* bars, unsigned g, int* err) {
+        const bool ok = __all_sync(kFull, mbar_wait(bars + g % NBUF, (g / NBUF) & 1, budget));
+        if (!ok && lane == 0) atomicOr(err, kErrTimeout);
+        return ok;
+    };
+    auto arrive_one = [&](unsigned long long* bar) {   // one arrival for the warp's accesses so far
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+    };
+    // Results of a finished chunk: RPI rows of SEG consecutive cells per store.
+    auto write_out = [&](unsigned g) {
+        const unsigned char* bp = buf((int)(g % NBUF));
+        const Hdr& h = *reinterpret_cast<const Hdr*>(bp + SM::off_h);
+        const T* w = reinterpret_cast<const T*>(bp);
+        const int kk = lane % SEG, r1 = lane / SEG, t0 = h.t0, nx = h.nx, rows = h.rows, dr = h.dr, dc = h.dc;
+        T* out = h.out;
+        constexpr int NI = SEG;   // 32 / RPI
+        T v[NI];
+#pragma unroll
+        for (int u = 0; u < NI; ++u) {
+            const int at = (r1 + u * RPI) * RS + kk;
+            v[u] = w[SM::W_SRC * SM::WIN + at];
+            if (DELTA) v[u] = (w[SM::W_IOLD * SM::WIN + at] + w[SM::W_SHIFT * SM::WIN + at]) + v[u];
+        }
+        if (rows == 32 && t0 >= 31 && t0 + SEG <= nx) {
+            T* o = out + r1 * dr + (t0 + kk - r1) * dc;
+            const int step = RPI * (dr - dc);
+#pragma unroll
+            for (int u = 0; u < NI; ++u) B::put(o + u * step, v[u]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < NI; ++u) {
+                const int r = r1 + u * RPI, c = t0 + kk - r;
+                if (r < rows && c >= 0 && c < nx) B::put(out + r * dr + c * dc, v[u]);
+            }
+        }
+    };
+
+    unsigned g = 0;   // chunks this warp has handled (buffer = g % NBUF)
+
+    auto load_warp = [&]() {
+        int next_static = pair * G + (int)blockIdx.x;
+        bool first = true;
+        // buffer of chunk g free: its previous chunk is written out
+        auto acquire = [&](int* err) {
+            if (g < NBUF) return true;
+            if (PREP) return wait_all(empty, g - NBUF, err);
+            if (!wait_all(done_b, g - NBUF, err)) return false;
+            write_out(g - NBUF);
+            __syncwarp();
+            return true;
+        };
+        for (;;) {
             // next unit; -1: none left, or an error was raised.  In a batch the
             // units of a problem that has stopped (converged or failed) are skipped.
             int t = -1, pp = 0, lt = 0;
@@ -510,92 +627,72 @@ sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
                     break;
                 }
             }
-            task = __shfl_sync(kFull, t, 0);
-            prob = __shfl_sync(kFull, pp, 0);
-            ltask = __shfl_sync(kFull, lt, 0);
+            const int task = __shfl_sync(kFull, t, 0), prob = __shfl_sync(kFull, pp, 0);
+            const int ltask = __shfl_sync(kFull, lt, 0);
             first = false;
-            if (task < 0) {   // end marker in the next buffer, then leave
+            if (task < 0) {   // end marker in the next buffer; without PREP the last chunks are still to be written
+                if (!acquire(c_err)) return;
                 const int b = (int)(g % NBUF);
-                if (g >= NBUF && !__all_sync(kFull, mbar_wait(empty + b, ((g / NBUF) - 1) & 1, budget))) {
-                    if (lane == 0) atomicOr(BATCH ? bt.err : a1.err, kErrTimeout);
-                    return;
-                }
-                if (lane == 0) *reinterpret_cast<volatile int*>(buf(b) + SM::off_h) = -1;
+                if (lane == 0) reinterpret_cast<Hdr*>(buf(b) + SM::off_h)->task = -1;
                 cp_async_mbar_arrive(full + b);
-                mbar_arrive(full + b);
+                arrive_one(full + b);
+                if (!PREP)
+                    for (unsigned q = g >= NBUF ? g - NBUF + 1 : 0; q < g; ++q) {
+                        if (!wait_all(done_b, q, c_err)) return;
+                        write_out(q);
+                    }
                 return;
             }
-        } else {
-            // the unit is in the header of its first chunk's buffer
-            const int b = (int)(g % NBUF);
-            if (!__all_sync(kFull, mbar_wait(full + b, (g / NBUF) & 1, budget))) {
-                if (lane == 0) atomicOr(BATCH ? bt.err : a1.err, kErrTimeout);
-                return;
-            }
-            const volatile int* h = reinterpret_cast<const volatile int*>(buf(b) + SM::off_h);
-            task = h[0];
-            if (task < 0) return;
-            prob = h[1];
-            ltask = h[2];
-        }
-        const SweepArgs<T>& a = BATCH ? bt.probs[prob] : a1;
-        const int nx = a.nx, ny = a.ny, K = a.K, nb = a.nb, nsteps = a.nsteps;
-        const int nchunks = (nsteps + SEG - 1) / SEG;
-        const int band = ltask / K;
-        const int s = ltask - band * K;
-        const bool xpos = a.qmu[s] >= 0.0, ypos = a.qeta[s] >= 0.0;
-        const int k = a.perm[s];
-        const int jl = band * 32 + lane;
-        const bool row_ok = jl < ny;
-        const int j = ypos ? jl : ny - 1 - jl;
-        T* Is = a.I + (size_t)s * a.N;
-        // cell of (band row r, sweep column c) = base0 + r * dr + c * dc
-        const bool full_rows = band * 32 + 32 <= ny;
-        const int dr = ypos ? nx : -nx, dc = xpos ? 1 : -1;
-        const int base0 = (ypos ? band * 32 : ny - 1 - band * 32) * nx + (xpos ? 0 : nx - 1);
-
-        if (copier) {
-            // ---------------------------------------------------- copy warp
+            const SweepArgs<T>& a = BATCH ? bt.probs[prob] : a1;
+            const int nx = a.nx, ny = a.ny, K = a.K, nb = a.nb, nsteps = a.nsteps;
+            const int nchunks = (nsteps + SEG - 1) / SEG;
+            const int band = ltask / K;
+            const int s = ltask - band * K;
+            const bool xpos = a.qmu[s] >= 0.0, ypos = a.qeta[s] >= 0.0;
+            const int k = a.perm[s];
+            const int rows = min(32, ny - band * 32);
+            // cell of (band row r, sweep column c) = base0 + r * dr + c * dc
+            const int dr = ypos ? nx : -nx, dc = xpos ? 1 : -1;
+            const int base0 = (ypos ? band * 32 : ny - 1 - band * 32) * nx + (xpos ? 0 : nx - 1);
             const T* wsrc[NW];
             wsrc[SM::W_SRC] = a.src + (size_t)s * a.src_stride;
-            if (!PRE) wsrc[SM::W_SIGT] = a.sigt;
-            if (PT) {
+            if constexpr (!PRE) wsrc[SM::W_SIGT] = a.sigt;
+            if constexpr (PT) {
                 wsrc[SM::W_SHIFT] = a.shift;
                 wsrc[SM::W_IOLD] = a.iold + (size_t)s * a.N;
             }
-            if (ADJ) {
+            if constexpr (ADJ) {
                 wsrc[SM::W_SHIFT] = a.ax;
                 wsrc[SM::W_IOLD] = a.ay;
             }
-            if (DELTA) {   // residual and stored intensity of this ordinate, correction per cell
+            if constexpr (DELTA) {   // residual and stored intensity of this ordinate, correction per cell
                 wsrc[SM::W_SRC] = a.src + (size_t)s * a.N;
                 wsrc[SM::W_SHIFT] = a.shift;
                 wsrc[SM::W_IOLD] = a.iold + (size_t)s * a.N;
             }
             const T* arow = a.acoef + (size_t)s * nx;
-            const double* rrow = PRE ? a.rsw + ((size_t)s * nb + band) * (size_t)a.nsteps * 32 : nullptr;
+            const double* rrow = PRE ? a.rsw + ((size_t)s * nb + band) * (size_t)nsteps * 32 : nullptr;
             T* edge_in = band > 0 ? a.edge + ((size_t)s * nb + band - 1) * nx : nullptr;
+            T bj = T(0), wall = T(0);   // this lane's row: |eta|/dy, the intensity entering through the wall
+            if (lane < rows) {
+                const int j = ypos ? band * 32 + lane : ny - 1 - band * 32 - lane;
+                bj = a.bcoef[(size_t)s * ny + j];
+                if (a.inflow) wall = (T)a.inflow[(size_t)(xpos ? j : ny + j) * K + k];
+            }
+            const int kk = lane % SEG, r1 = lane / SEG;
             for (int m = 0; m < nchunks; ++m, ++g) {
+                if (!acquire(a.err)) return;
                 const int b = (int)(g % NBUF);
-                if (g >= NBUF) {
-                    const bool ok = __all_sync(kFull, mbar_wait(empty + b, ((g / NBUF) - 1) & 1, budget));
-                    if (!ok) {
-                        if (lane == 0) atomicOr(a.err, kErrTimeout);
-                        cp_async_wait_all();
-                        return;
-                    }
-                }
                 unsigned char* bp = buf(b);
                 T* wb = reinterpret_cast<T*>(bp);
+                T* ab = reinterpret_cast<T*>(bp + SM::off_a);
                 const int t0 = m * SEG;
-                constexpr int RPI = 32 / SEG;   // rows per copy instruction
-                const int kk = lane % SEG;
-                if (full_rows && t0 >= 31 && t0 + SEG <= nx) {
+                // row r of the band needs columns t0 - r .. t0 - r + SEG - 1
+                if (rows == 32 && t0 >= 31 && t0 + SEG <= nx) {
                     // interior chunk: every row window lies inside the mesh
-                    const int r = lane / SEG;
-                    int cell = base0 + r * dr + (t0 + kk - r) * dc;
+                    int cell = base0 + r1 * dr + (t0 + kk - r1) * dc;
                     const int dcell = RPI * (dr - dc);
-                    T* dst = wb + r * RS + kk;
+                    T* dst = wb + r1 * RS + kk;
 #pragma unroll
                     for (int r0 = 0; r0 < 32; r0 += RPI) {
 #pragma unroll
@@ -603,218 +700,258 @@ sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
                         cell += dcell;
                         dst += RPI * RS;
                     }
-                    T* ab = reinterpret_cast<T*>(bp + SM::off_a);
-                    for (int u = lane; u < SEG + 31; u += 32)
-                        cp_async<sizeof(T)>(ab + u, arow + (xpos ? t0 - 31 + u : nx - 1 - (t0 - 31 + u)));
+                    const T* ap = arow + (xpos ? t0 - 31 : nx - 1 - (t0 - 31));
+                    for (int u = lane; u < SEG + 31; u += 32) cp_async<sizeof(T)>(ab + u, ap + u * dc);
                 } else {
-                    // row r of the band needs columns t0 - r .. t0 - r + SEG - 1
-#pragma unroll 4
-                    for (int r0 = 0; r0 < 32; r0 += RPI) {
-                        const int r = r0 + lane / SEG;
-                        const int jr = band * 32 + r;
-                        const int c = t0 + kk - r;
-                        if (jr < ny && c >= 0 && c < nx) {
-                            const size_t cell = (size_t)(ypos ? jr : ny - 1 - jr) * nx + (xpos ? c : nx - 1 - c);
+                    // at the walls: the nearest cell's data where the window leaves the mesh
 #pragma unroll
-                            for (int w = 0; w < NW; ++w) cp_async<sizeof(T)>(wb + w * SM::WIN + r * RS + kk, wsrc[w] + cell);
-                        }
+                    for (int r0 = 0; r0 < 32; r0 += RPI) {
+                        const int r = r0 + r1;
+                        const int c = min(max(t0 + kk - r, 0), nx - 1);
+                        const int cell = base0 + min(r, rows - 1) * dr + c * dc;
+#pragma unroll
+                        for (int w = 0; w < NW; ++w) cp_async<sizeof(T)>(wb + w * SM::WIN + r * RS + kk, wsrc[w] + cell);
                     }
-                    T* ab = reinterpret_cast<T*>(bp + SM::off_a);
                     for (int u = lane; u < SEG + 31; u += 32) {
-                        const int c = t0 - 31 + u;
-                        if (c >= 0 && c < nx) cp_async<sizeof(T)>(ab + u, arow + (xpos ? c : nx - 1 - c));
+                        const int c = min(max(t0 - 31 + u, 0), nx - 1);
+                        cp_async<sizeof(T)>(ab + u, arow + (xpos ? c : nx - 1 - c));
                     }
                 }
-                if (PRE) {
+                if constexpr (PRE) {
                     const int nv = min(SEG, nsteps - t0) * 32;   // doubles, multiple of 32
                     double* rb = reinterpret_cast<double*>(bp + SM::off_r);
-                    for (int v = 2 * lane; v < nv; v += 64) cp_async<16>(rb + v, rrow + (size_t)t0 * 32 + v);
+                    const double* rp = rrow + (size_t)t0 * 32;
+#pragma unroll
+                    for (int v = 0; v < SEG * 32; v += 64)
+                        if (v + 2 * lane < nv) cp_async<16>(rb + v + 2 * lane, rp + v + 2 * lane);
                 }
                 cp_async_mbar_arrive(full + b);
-                // south values of lane 0 for columns t0 .. t0 + SEG - 1
-                T ev = T(0);
-                const bool need = lane < SEG && t0 + lane < nx;
-                if (band == 0) {
-                    if (need && a.inflow) {
-                        const int c = t0 + lane;
-                        const int i = xpos ? c : nx - 1 - c;
-                        const int f = ypos ? 2 * ny + i : 2 * ny + nx + i;
-                        ev = (T)a.inflow[(size_t)f * K + k];
+                if (m == 0) {
+                    T* cx = reinterpret_cast<T*>(bp + SM::off_c);
+                    cx[lane] = bj;
+                    cx[32 + lane] = wall;
+                }
+                if (lane == 0) {
+                    Hdr& h = *reinterpret_cast<Hdr*>(bp + SM::off_h);
+                    h.task = task;
+                    h.nchunks = nchunks;
+                    h.nx = nx;
+                    h.rows = rows;
+                    h.out = a.I + (size_t)s * a.N + base0;
+                    h.eo = a.edge + ((size_t)s * nb + band) * nx;
+                    h.err = a.err;
+                    h.t0 = t0;
+                    h.dr = dr;
+                    h.dc = dc;
+                    h.put_edge = band < nb - 1;
+                    h.ei = edge_in;
+                    h.in = nullptr;
+                    if (a.inflow) {   // sweep column 0's face of the wall below, then along the row
+                        h.in = a.inflow + (size_t)((ypos ? 2 * ny : 2 * ny + nx) + (xpos ? 0 : nx - 1)) * K + k;
+                        h.in_step = xpos ? K : -K;
                     }
-                } else {
-                    bool have = !need;
+                    if (ADJ && m == 0) {
+                        const double ws = a.qw[s];
+                        h.cw = (T)ws;
+                        h.cm = (T)(-ws * a.qmu[s]);
+                        h.ce = (T)(-ws * a.qeta[s]);
+                    }
+                }
+                arrive_one(full + b);
+            }
+        }
+    };
+
+    // South values of lane 0: per chunk the inflow (band 0) or the band below's
+    // last-row results, polled until they are written.
+    auto south_warp = [&]() {
+        using U = typename B::U;
+        int* err = c_err;
+        for (;;) {
+            if (!wait_all(full, g, err)) return;
+            const Hdr& h = *reinterpret_cast<const Hdr*>(buf((int)(g % NBUF)) + SM::off_h);
+            if (h.task < 0) {
+                arrive_one(ready + g % NBUF);
+                return;
+            }
+            const int nchunks = h.nchunks, nx = h.nx;
+            T* const ei = h.ei;
+            const double* const in = h.in;
+            const long long in_step = h.in_step;
+            err = h.err;
+            for (int m = 0; m < nchunks; ++m, ++g) {
+                const int c = m * SEG + lane;
+                const bool need = lane < SEG && c < nx;
+                U u = B::empty;
+                T ev = T(0);
+                if (need) {   // in flight during the wait
+                    if (ei) u = B::load(ei + c);
+                    else if (in) ev = (T)in[c * in_step];
+                }
+                if (m > 0 && !wait_all(full, g, err)) return;
+                if (ei) {
                     const long long start = clock64();
-                    for (;;) {
-                        if (!have) {
-                            const typename B::U u = B::load(edge_in + t0 + lane);
-                            if (u != B::empty) {
-                                have = true;
-                                ev = B::value(u);
-                            }
-                        }
-                        if (__all_sync(kFull, have)) break;
+                    while (!__all_sync(kFull, !need || u != B::empty)) {
                         if (__any_sync(kFull, clock64() - start > budget)) {   // warp-uniform exit
-                            if (lane == 0) atomicOr(a.err, kErrTimeout);
-                            cp_async_wait_all();
+                            if (lane == 0) atomicOr(err, kErrTimeout);
                             return;
                         }
-                        __nanosleep(20);
+                        if (need && u == B::empty) u = B::load(ei + c);
                     }
+                    if (need) ev = B::value(u);
                 }
-                if (lane < SEG) reinterpret_cast<T*>(bp + SM::off_e)[lane] = ev;
-                if (lane == 0) {
-                    volatile int* h = reinterpret_cast<volatile int*>(bp + SM::off_h);
-                    h[0] = task;
-                    h[1] = prob;
-                    h[2] = ltask;
-                }
-                mbar_arrive(full + b);
+                const int b = (int)(g % NBUF);
+                if (lane < SEG) reinterpret_cast<T*>(buf(b) + SM::off_e)[lane] = ev;
+                arrive_one(ready + b);
             }
             // every value of the upstream hand-off row has been taken:
             // mark it unwritten for the next sweep
-            if (band > 0)
-                for (int c = lane; c < nx; c += 32) B::clear(edge_in + c);
-        } else {
-            // ------------------------------------------------- compute warp
-            const T bj = row_ok ? a.bcoef[(size_t)s * ny + j] : T(0);
-            T cw = T(0), cm = T(0), ce = T(0);   // adjoint source w (a - mu bx - eta by)
-            if (ADJ) {
-                const double ws = a.qw[s];
-                cw = (T)ws;
-                cm = (T)(-ws * a.qmu[s]);
-                ce = (T)(-ws * a.qeta[s]);
+            if (ei)
+                for (int c = lane; c < nx; c += 32) B::clear(ei + c);
+        }
+    };
+
+    auto prep_warp = [&]() {
+        unsigned written = 0;   // chunks written out
+        int* err = c_err;
+        auto write_next = [&]() {
+            if (!wait_all(done_b, written, err)) return false;
+            write_out(written);
+            arrive_one(empty + written % NBUF);
+            ++written;
+            return true;
+        };
+        for (;;) {
+            if (!wait_all(full, g, err)) return;
+            const Hdr& h0 = *reinterpret_cast<const Hdr*>(buf((int)(g % NBUF)) + SM::off_h);
+            if (h0.task < 0) {
+                arrive_one(ready + g % NBUF);
+                while (written < g)
+                    if (!write_next()) return;
+                return;
             }
-            T IW = T(0);
-            if (row_ok && a.inflow) IW = (T)a.inflow[(size_t)(xpos ? j : ny + j) * K + k];
-            T Iprev = T(0);
-            T* eo = a.edge + ((size_t)s * nb + band) * nx;   // this band's last row, by column
-            const bool put_edge = lane == 31 && band < nb - 1;
+            const int nchunks = h0.nchunks;
+            err = h0.err;
+            const T cw = h0.cw, cm = h0.cm, ce = h0.ce;
+            const T bj = reinterpret_cast<const T*>(buf((int)(g % NBUF)) + SM::off_c)[lane];
             for (int m = 0; m < nchunks; ++m, ++g) {
-                const int b = (int)(g % NBUF);
-                const bool ok = __all_sync(kFull, mbar_wait(full + b, (g / NBUF) & 1, budget));
-                if (!ok) {
-                    if (lane == 0) atomicOr(a.err, kErrTimeout);
-                    return;
-                }
-                unsigned char* bp = buf(b);
-                // the lane's row; with STAGE its source slots collect the results
-                T* wb = reinterpret_cast<T*>(bp) + lane * RS;
+                if (m > 0 && !wait_all(full, g, err)) return;
+                unsigned char* bp = buf((int)(g % NBUF));
+                T* w = reinterpret_cast<T*>(bp) + lane * RS;
                 const T* ab = reinterpret_cast<const T*>(bp + SM::off_a) + 31 - lane;
-                const double* rb = reinterpret_cast<const double*>(bp + SM::off_r) + lane;
-                const T* ein = reinterpret_cast<const T*>(bp + SM::off_e);
+                float d[PRE ? 1 : SEG];
+                unsigned dlo = ~0u, dhi = 0u;
+#pragma unroll
+                for (int tt = 0; tt < SEG; ++tt) {
+                    T sv = w[SM::W_SRC * SM::WIN + tt];
+                    if (ADJ) sv = fma(cm, w[SM::W_SHIFT * SM::WIN + tt], fma(ce, w[SM::W_IOLD * SM::WIN + tt], cw * sv));
+                    T sh = T(0);
+                    if (PT) {
+                        sh = w[SM::W_SHIFT * SM::WIN + tt];
+                        sv = fma(sh, w[SM::W_IOLD * SM::WIN + tt], sv);
+                    }
+                    if (ADJ || PT) w[SM::W_SRC * SM::WIN + tt] = sv;
+                    if constexpr (!PRE) {
+                        d[tt] = w[SM::W_SIGT * SM::WIN + tt] + ab[tt] + bj;
+                        if (PT) d[tt] += sh;
+                        dlo = min(dlo, __float_as_uint(d[tt]));
+                        dhi = max(dhi, __float_as_uint(d[tt]));
+                    }
+                }
+                if constexpr (!PRE) {
+                    const bool plain = dlo >= kRcpLo && dhi <= kRcpHi;
+#pragma unroll
+                    for (int tt = 0; tt < SEG; ++tt)
+                        w[SM::W_SIGT * SM::WIN + tt] = plain ? rcp_newton(d[tt]) : 0.f;
+                    if (!plain) {
+#pragma unroll
+                        for (int tt = 0; tt < SEG; ++tt) w[SM::W_SIGT * SM::WIN + tt] = __frcp_rn(d[tt]);
+                    }
+                }
+                arrive_one(ready + g % NBUF);
+                if (g >= 2 && !write_next()) return;
+            }
+        }
+    };
+
+    auto compute_warp = [&]() {
+        unsigned long long* in = ready;
+        for (;;) {
+            if (!wait_all(in, g, c_err)) return;
+            const unsigned char* b0 = buf((int)(g % NBUF));
+            const Hdr& h = *reinterpret_cast<const Hdr*>(b0 + SM::off_h);
+            if (h.task < 0) return;
+            const int nchunks = h.nchunks, nx = h.nx;
+            const bool full_rows = h.rows == 32, put_edge = lane == 31 && h.put_edge;
+            T* eo = h.eo;
+            int* err = h.err;
+            const T* cx = reinterpret_cast<const T*>(b0 + SM::off_c);
+            const T bj = cx[lane], wall = cx[32 + lane];
+            T IW = wall, Iprev = T(0);
+            T sv_n = T(0), ai_n = T(0), r_n = T(0), e_n = T(0);   // next step's operands, read one step ahead
+            bool ahead = false;                                   // ... of the next chunk already
+            auto operands = [&](const unsigned char* bp, int tt) {
+                const T* w = reinterpret_cast<const T*>(bp) + lane * RS + tt;
+                sv_n = w[SM::W_SRC * SM::WIN];
+                ai_n = (reinterpret_cast<const T*>(bp + SM::off_a) + 31 - lane)[tt];
+                if constexpr (PRE) r_n = (reinterpret_cast<const T*>(bp + SM::off_r) + lane)[tt * 32];
+                else r_n = w[SM::W_SIGT * SM::WIN];
+                e_n = reinterpret_cast<const T*>(bp + SM::off_e)[tt];
+            };
+            for (int m = 0; m < nchunks; ++m, ++g) {
+                if (!ahead) {
+                    if (m > 0 && !wait_all(in, g, err)) return;
+                    operands(buf((int)(g % NBUF)), 0);
+                }
+                ahead = false;
+                unsigned char* bp = buf((int)(g % NBUF));
+                T* res = reinterpret_cast<T*>(bp) + lane * RS;   // the source slots collect the results
                 const int t0 = m * SEG;
-                if (full_rows && t0 >= 31 && t0 + SEG <= nx) {
-                    // interior chunk: every lane updates a cell at every step
-                    T* Ic = Is + base0 + lane * dr + (t0 - lane) * dc;
-                    T* ec = eo + (t0 - 31);
-                    // the step's source, column coefficient and 1/d depend only on
-                    // the chunk's data: they are formed one step ahead, so that
-                    // only the two upwind FMAs and the 1/d multiply wait on the
-                    // previous step
-                    auto operands = [&](int tt, T& sv, T& ai, T& rinv) {
-                        sv = wb[SM::W_SRC * SM::WIN + tt];
-                        if (ADJ) sv = fma(cm, wb[SM::W_SHIFT * SM::WIN + tt], fma(ce, wb[SM::W_IOLD * SM::WIN + tt], cw * sv));
-                        ai = ab[tt];
-                        if (PRE) {
-                            if (PT) sv = fma(wb[SM::W_SHIFT * SM::WIN + tt], wb[SM::W_IOLD * SM::WIN + tt], sv);
-                            rinv = (T)rb[tt * 32];
-                        } else {
-                            T d = wb[SM::W_SIGT * SM::WIN + tt] + ai + bj;
-                            if (PT) {
-                                const T sh = wb[SM::W_SHIFT * SM::WIN + tt];
-                                sv = fma(sh, wb[SM::W_IOLD * SM::WIN + tt], sv);
-                                d += sh;
-                            }
-                            rinv = rcp_t(d);
-                        }
-                    };
-                    T sv_n, ai_n, rinv_n;
-                    operands(0, sv_n, ai_n, rinv_n);
+                auto steps = [&](auto wall_chunk) {
+                    constexpr bool WALL = decltype(wall_chunk)::value;
 #pragma unroll
                     for (int tt = 0; tt < SEG; ++tt) {
-                        const T sv = sv_n, ai = ai_n, rinv = rinv_n;
-                        if (tt + 1 < SEG) operands(tt + 1, sv_n, ai_n, rinv_n);
+                        const T sv = sv_n, ai = ai_n, rinv = r_n, e = e_n;
+                        if (tt + 1 < SEG) operands(bp, tt + 1);
+                        else if (m + 1 < nchunks) {
+                            // a look at the next chunk while this step's chain runs; not a wait:
+                            // the band above may need this step first
+                            const unsigned gn = g + 1;
+                            ahead = __all_sync(kFull, mbar_test(in + gn % NBUF, (gn / NBUF) & 1));
+                            if (ahead) operands(buf((int)(gn % NBUF)), 0);
+                        }
+                        if (WALL && t0 + tt == lane) IW = wall;   // the lane's first column
                         // lane l gets lane l-1's previous result; lane 0 the south value
-                        const T e = ein[tt];
                         const T Isouth = __shfl_sync(kFull, lane == 31 ? e : Iprev, (lane + 31) & 31);
                         T acc = fma(ai, IW, sv);
                         acc = fma(bj, Isouth, acc);
                         const T Inew = acc * rinv;
                         IW = Inew;
                         Iprev = Inew;
-                        const T out = DELTA ? (wb[SM::W_IOLD * SM::WIN + tt] + wb[SM::W_SHIFT * SM::WIN + tt]) + Inew : Inew;
-                        if constexpr (STAGE) wb[SM::W_SRC * SM::WIN + tt] = out;   // the slot just read
-                        else B::put(Ic + tt * dc, out);
-                        if (put_edge) B::store(ec + tt, Inew);
+                        res[SM::W_SRC * SM::WIN + tt] = Inew;
+                        const int c = t0 + tt - 31;
+                        if (put_edge && (!WALL || (c >= 0 && c < nx))) B::store(eo + c, Inew);
                     }
-                } else {
-#pragma unroll 4
-                    for (int tt = 0; tt < SEG; ++tt) {
-                        const int t = t0 + tt;
-                        if (t >= nsteps) break;
-                        const T e = ein[tt];
-                        const T Isouth = __shfl_sync(kFull, lane == 31 ? e : Iprev, (lane + 31) & 31);
-                        const int c = t - lane;
-                        T Inew = T(0);
-                        if (row_ok && c >= 0 && c < nx) {
-                            T sv = wb[SM::W_SRC * SM::WIN + tt];
-                            if (ADJ) sv = fma(cm, wb[SM::W_SHIFT * SM::WIN + tt], fma(ce, wb[SM::W_IOLD * SM::WIN + tt], cw * sv));
-                            const T ai = ab[tt];
-                            T rinv;
-                            if (PRE) {
-                                if (PT) sv = fma(wb[SM::W_SHIFT * SM::WIN + tt], wb[SM::W_IOLD * SM::WIN + tt], sv);
-                                    rinv = (T)rb[tt * 32];
-                            } else {
-                                T d = wb[SM::W_SIGT * SM::WIN + tt] + ai + bj;
-                                if (PT) {
-                                    const T sh = wb[SM::W_SHIFT * SM::WIN + tt];
-                                    sv = fma(sh, wb[SM::W_IOLD * SM::WIN + tt], sv);
-                                    d += sh;
-                                }
-                                rinv = rcp_t(d);
-                            }
-                            T acc = fma(ai, IW, sv);
-                            acc = fma(bj, Isouth, acc);
-                            Inew = acc * rinv;
-                            IW = Inew;
-                            const T out =
-                                DELTA ? (wb[SM::W_IOLD * SM::WIN + tt] + wb[SM::W_SHIFT * SM::WIN + tt]) + Inew : Inew;
-                            if constexpr (STAGE) wb[SM::W_SRC * SM::WIN + tt] = out;
-                            else B::put(Is + base0 + lane * dr + c * dc, out);
-                            if (put_edge) B::store(eo + c, Inew);
-                        }
-                        Iprev = Inew;
-                    }
-                }
-                if constexpr (STAGE) {
-                    // write the chunk's results out row by row: RPI rows of SEG
-                    // consecutive cells per store instruction instead of one
-                    // cell of each of 32 rows
-                    __syncwarp();
-                    constexpr int RPI = 32 / SEG;
-                    const int kk = lane % SEG;
-                    const T* stage = reinterpret_cast<const T*>(bp);
-#pragma unroll 4
-                    for (int r0 = 0; r0 < 32; r0 += RPI) {
-                        const int r = r0 + lane / SEG;
-                        const int c = t0 + kk - r;
-                        if (band * 32 + r < ny && c >= 0 && c < nx)
-                            B::put(Is + base0 + r * dr + c * dc, stage[r * RS + kk]);
-                    }
-                    __syncwarp();
-                }
-                mbar_arrive(empty + b);
+                };
+                if (full_rows && t0 >= 31 && t0 + SEG <= nx) steps(std::false_type{});
+                else steps(std::true_type{});
+                arrive_one(done_b + g % NBUF);
             }
         }
-    }
     };
-    body();
-    if (copier) cp_async_wait_all();
+
+    if (!cta_stop) {
+        if (role == 0) compute_warp();
+        else if (role == 1) load_warp();
+        else if (role == 2) south_warp();
+        else prep_warp();
+    }
+    if (role == 1) cp_async_wait_all();
     // the launch's last warp to leave re-arms the counters for the next launch
     __syncwarp();
     if (lane == 0) {
         __threadfence();
-        if (atomicAdd(c_exits, 1u) == (unsigned)G * (unsigned)(2 * SM::PAIRS) - 1u) {
+        if (atomicAdd(c_exits, 1u) == (unsigned)G * (unsigned)(SM::WARPS * SM::PAIRS) - 1u) {
             *c_tasks = 0u;
             *c_arrived = 0u;
             *c_mode = 0;
@@ -1094,16 +1231,6 @@ int grid_for(long long n, int block, int cap)
     return (int)g;
 }
 
-template <typename T, int MODE, bool BATCH = false>
-size_t sweep_smem();
-
-// Threads of one sweep CTA of this variant (its pairs x 64).
-template <typename T, int MODE, bool BATCH = false>
-constexpr int sweep_threads()
-{
-    return SweepSmem<T, sweep_xw(MODE), sizeof(T) == 8, BATCH>::PAIRS * 64;
-}
-
 template <typename T, int MODE>
 SweepArgs<T> sweep_args(const Plan& P)
 {
@@ -1150,11 +1277,11 @@ SweepArgs<T> sweep_args(const Plan& P)
     return a;
 }
 
-template <typename T, int MODE, bool PRE>
+template <typename T, int MODE>
 cudaError_t launch_sweep_t(Plan& P, cudaStream_t st)
 {
     const SweepArgs<T> a = sweep_args<T, MODE>(P);
-    sweep_kernel<T, MODE, PRE, false><<<P.sweep_grid, sweep_threads<T, MODE>(), sweep_smem<T, MODE>(), st>>>(a, SweepBatch<T>{});
+    sweep_kernel<T, MODE, false><<<P.sweep_grid, SweepSmem<T, MODE>::THREADS, SweepSmem<T, MODE>::bytes, st>>>(a, SweepBatch<T>{});
     return cudaGetLastError();
 }
 
@@ -1175,7 +1302,7 @@ cudaError_t launch_sweep_batch_t(const BatchTables& bt, cudaStream_t st)
     b.mode = &bt.status->sweep_mode;
     b.err = &bt.status->error;
     b.wait_cycles = bt.wait_cycles;
-    sweep_kernel<T, MODE, sizeof(T) == 8, true><<<bt.sweep_grid, sweep_threads<T, MODE, true>(), sweep_smem<T, MODE, true>(), st>>>(
+    sweep_kernel<T, MODE, true><<<bt.sweep_grid, SweepSmem<T, MODE>::THREADS, SweepSmem<T, MODE>::bytes, st>>>(
         SweepArgs<T>{}, b);
     return cudaGetLastError();
 }
@@ -1256,17 +1383,10 @@ cudaError_t launch_moments_t(const Plan& P, bool with_F, bool with_P, double* rh
 }
 
 template <typename T, int MODE, bool BATCH>
-size_t sweep_smem()
-{
-    return SweepSmem<T, sweep_xw(MODE), sizeof(T) == 8, BATCH>::bytes;
-}
-
-
-template <typename T, int MODE, bool BATCH>
 cudaError_t sweep_attr()
 {
-    return cudaFuncSetAttribute(sweep_kernel<T, MODE, sizeof(T) == 8, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sweep_smem<T, MODE, BATCH>());
+    return cudaFuncSetAttribute(sweep_kernel<T, MODE, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)SweepSmem<T, MODE>::bytes);
 }
 
 // Raises the dynamic shared-memory limit of fn to at least `bytes` (never
@@ -1297,13 +1417,6 @@ cudaError_t prepare_t(int K)
             (e = sweep_attr<T, kSrcPlain, true>()) != cudaSuccess ||
             (e = sweep_attr<T, kSrcPseudoTime, true>()) != cudaSuccess)
             first = e;
-        if constexpr (sizeof(T) == 8) {   // the FP64 throughput form
-            if (first == cudaSuccess &&
-                (e = cudaFuncSetAttribute(sweep_kernel<double, kSrcPlain, true, false, true>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sweep_smem<double, kSrcPlain, true>())) != cudaSuccess)
-                first = e;
-        }
     });
     if (first != cudaSuccess) return first;
     const size_t ms = moments_smem<T>(K);
@@ -1322,19 +1435,8 @@ template <typename T, int MODE, bool BATCH>
 int sweep_occupancy()
 {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, MODE, sizeof(T) == 8, BATCH>,
-                                                      sweep_threads<T, MODE, BATCH>(), sweep_smem<T, MODE, BATCH>()) != cudaSuccess)
-        return 0;
-    return n;
-}
-
-template <int MODE, bool WIDE>
-int sweep_fp64_occupancy()
-{
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<double, MODE, true, false, WIDE>,
-                                                      sweep_threads<double, MODE, WIDE>(),
-                                                      sweep_smem<double, MODE, WIDE>()) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, MODE, BATCH>,
+                                                      SweepSmem<T, MODE>::THREADS, SweepSmem<T, MODE>::bytes) != cudaSuccess)
         return 0;
     return n;
 }
@@ -1423,15 +1525,6 @@ cudaError_t launch_source_from(const Plan& P, const double* rho_in, cudaStream_t
     return cudaGetLastError();
 }
 
-// The FP64 sweep's throughput form pays when every pair has several long
-// units to run (1024^2 S16: 4608 units, sweep 1.32 -> 1.09 ms); with fewer
-// units than two waves of the 8-pair form the band hand-off latency
-// dominates and per-result stores are faster (256^2 S12: 672 units).
-bool sweep_wide(const Plan& P)
-{
-    return (long long)P.K * P.nb >= 2LL * P.sweep_grid * 8;
-}
-
 cudaError_t launch_sweep(Plan& P, cudaStream_t st)
 {
     if (P.pt && P.X && !P.fp32) {
@@ -1441,14 +1534,8 @@ cudaError_t launch_sweep(Plan& P, cudaStream_t st)
         SweepArgs<double> a = sweep_args<double, kSrcPlain>(P);
         a.src = P.X;
         a.src_stride = P.N;
-        if (sweep_wide(P)) {   // throughput form: 12 pairs, staged write-out (same bits)
-            sweep_kernel<double, kSrcPlain, true, false, true>
-                <<<P.sweep_grid, sweep_threads<double, kSrcPlain, true>(), sweep_smem<double, kSrcPlain, true>(), st>>>(
-                    a, SweepBatch<double>{});
-            return cudaGetLastError();
-        }
-        sweep_kernel<double, kSrcPlain, true, false>
-            <<<P.sweep_grid, sweep_threads<double, kSrcPlain>(), sweep_smem<double, kSrcPlain>(), st>>>(a, SweepBatch<double>{});
+        sweep_kernel<double, kSrcPlain, false>
+            <<<P.sweep_grid, SweepSmem<double, kSrcPlain>::THREADS, SweepSmem<double, kSrcPlain>::bytes, st>>>(a, SweepBatch<double>{});
         return cudaGetLastError();
     }
     if (P.fp32 && P.pt && P.X_f) {
@@ -1459,38 +1546,37 @@ cudaError_t launch_sweep(Plan& P, cudaStream_t st)
         a.src = P.X_f;
         a.src_stride = P.N;
         a.sigt = P.sigt_d;
-        sweep_kernel<float, kSrcPlain, false, false>
-            <<<P.sweep_grid, sweep_threads<float, kSrcPlain>(), sweep_smem<float, kSrcPlain>(), st>>>(a, SweepBatch<float>{});
+        sweep_kernel<float, kSrcPlain, false>
+            <<<P.sweep_grid, SweepSmem<float, kSrcPlain>::THREADS, SweepSmem<float, kSrcPlain>::bytes, st>>>(a, SweepBatch<float>{});
         return cudaGetLastError();
     }
     if (P.fp32) {
-        return P.pt ? launch_sweep_t<float, kSrcPseudoTime, false>(P, st)
-                    : launch_sweep_t<float, kSrcPlain, false>(P, st);
+        return P.pt ? launch_sweep_t<float, kSrcPseudoTime>(P, st)
+                    : launch_sweep_t<float, kSrcPlain>(P, st);
     }
-    return P.pt ? launch_sweep_t<double, kSrcPseudoTime, true>(P, st) : launch_sweep_t<double, kSrcPlain, true>(P, st);
+    return P.pt ? launch_sweep_t<double, kSrcPseudoTime>(P, st) : launch_sweep_t<double, kSrcPlain>(P, st);
 }
 
 cudaError_t launch_delta_sweep(Plan& P, cudaStream_t st)
 {
-    return P.fp32 ? launch_sweep_t<float, kSrcDelta, false>(P, st) : launch_sweep_t<double, kSrcDelta, true>(P, st);
+    return P.fp32 ? launch_sweep_t<float, kSrcDelta>(P, st) : launch_sweep_t<double, kSrcDelta>(P, st);
 }
 
 cudaError_t launch_adjoint_sweep(Plan& P, cudaStream_t st)
 {
-    return P.fp32 ? launch_sweep_t<float, kSrcAdjoint, false>(P, st) : launch_sweep_t<double, kSrcAdjoint, true>(P, st);
+    return P.fp32 ? launch_sweep_t<float, kSrcAdjoint>(P, st) : launch_sweep_t<double, kSrcAdjoint>(P, st);
 }
 
 template <typename T>
 cudaError_t launch_sweep_pt_into_t(Plan& P, const void* src, const void* iold, void* out, cudaStream_t st)
 {
-    constexpr bool PRE = sizeof(T) == 8;
     SweepArgs<T> a = sweep_args<T, kSrcPseudoTime>(P);
     a.src = static_cast<const T*>(src);
     a.iold = static_cast<const T*>(iold);
     a.I = static_cast<T*>(out);
     a.inflow = nullptr;
-    sweep_kernel<T, kSrcPseudoTime, PRE, false>
-        <<<P.sweep_grid, sweep_threads<T, kSrcPseudoTime>(), sweep_smem<T, kSrcPseudoTime>(), st>>>(a, SweepBatch<T>{});
+    sweep_kernel<T, kSrcPseudoTime, false>
+        <<<P.sweep_grid, SweepSmem<T, kSrcPseudoTime>::THREADS, SweepSmem<T, kSrcPseudoTime>::bytes, st>>>(a, SweepBatch<T>{});
     return cudaGetLastError();
 }
 
@@ -1609,7 +1695,7 @@ int sweep_max_active_blocks(int fp32, int pt)
     return std::min({sweep_occupancy<double, kSrcPlain, false>(), sweep_occupancy<double, kSrcPseudoTime, false>(),
                      sweep_occupancy<double, kSrcAdjoint, false>(), sweep_occupancy<double, kSrcDelta, false>(),
                      sweep_occupancy<double, kSrcPlain, true>(),
-                     sweep_occupancy<double, kSrcPseudoTime, true>(), sweep_fp64_occupancy<kSrcPlain, true>()});
+                     sweep_occupancy<double, kSrcPseudoTime, true>()});
 }
 
 }  // namespace gsis
