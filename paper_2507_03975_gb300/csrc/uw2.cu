@@ -14,8 +14,9 @@
 //    (Eq. (Iij)), the inflow on incoming boundary faces;
 //  * R = S - sigma_t I_i - mu (I_E - I_W)/dx - eta (I_N - I_S)/dy
 //    (Eq. (RTE_d_res), steady, per unit volume).
-// The residual kernel is tiled (a cell tile plus halo per CTA, each limited
-// gradient computed once); the boundary flux reads global memory.
+// The residual kernel marches (a warp per ordinate and column strip, each
+// limited gradient and face value formed once); the boundary flux reads
+// global memory.
 #include <cuda_runtime.h>
 
 #include "gsis_internal.cuh"
@@ -86,118 +87,136 @@ __device__ __forceinline__ void limited_gradient(const Uw2Args<T>& a, const T* I
                           a.limiter, gx, gy);
 }
 
-// Tiled residual: a CTA takes a TX x TY tile of cells and DPB ordinates; per
-// ordinate the intensities of the tile and a two-cell halo go to shared
-// memory, the limited gradients of the tile and a one-cell halo are computed
-// once, then every tile cell assembles its residual from its own and its
-// upwind neighbours' reconstructions.
-constexpr int kTX = 32, kTY = 8, kLX = kTX + 4, kLY = kTY + 4, kGX = kTX + 2, kGY = kTY + 2;
-constexpr int kDPB = 8;
+// The Barth-Jespersen factor from the differences to the neighbours, east,
+// west (negated), ahead, behind (negated; 0 where there is none) and the face
+// changes hx/2 G_x, hy/2 G_y: false where the limiter does not act.  Rounding is
+// monotone, so the largest difference is the difference to the largest value.
+// In double on the bits: numbers of which one is >= 0 are ordered like their
+// bits as signed integers; a comparison, a sign change or a magnitude would be
+// an FP64 pipe instruction each (19 cycles per SM).
+__device__ __forceinline__ bool limit(double dE, double dWn, double dA, double dBn, double cx, double cy, double& psi)
+{
+    constexpr long long S = 1ll << 63;
+    const long long e = __double_as_longlong(dE), w = __double_as_longlong(dWn) ^ S, a = __double_as_longlong(dA),
+                    b = __double_as_longlong(dBn) ^ S;
+    const long long up = max(max(max(e, w), max(a, b)), 0ll), dn = max(max(max(e ^ S, w ^ S), max(a ^ S, b ^ S)), 0ll);
+    const long long dm = max(__double_as_longlong(cx) & ~S, __double_as_longlong(cy) & ~S), room = min(up, dn);
+    if (!(room < dm)) return false;
+    psi = __longlong_as_double(room) / __longlong_as_double(dm);
+    return true;
+}
+
+__device__ __forceinline__ bool limit(float dE, float dWn, float dA, float dBn, float cx, float cy, float& psi)
+{
+    const float up = fmaxf(fmaxf(fmaxf(dE, -dWn), fmaxf(dA, -dBn)), 0.f);
+    const float dn = fmaxf(fmaxf(fmaxf(-dE, dWn), fmaxf(-dA, dBn)), 0.f);
+    const float dm = fmaxf(fabsf(cx), fabsf(cy)), room = fminf(up, dn);
+    if (!(dm > 0.f) || !(room < dm)) return false;
+    psi = room / dm;
+    return true;
+}
+
+// x / h with y = 1/h correctly rounded: the quotient x y corrected by its exact
+// residual is the correctly rounded one (Markstein 1990, "Computation of
+// elementary functions on the IBM RISC System/6000"), so the bits of x / h, in
+// three FP64 operations.
+__device__ __forceinline__ double div_by(double x, double h, double y)
+{
+    const double q = x * y;
+    return fma(fma(-q, h, x), y, q);
+}
+__device__ __forceinline__ float div_by(float x, float h, float) { return x / h; }
+
+// Residual, one warp per ordinate, 29 columns and kUwRows rows.  The FP64
+// pipe bounds it, so every quantity that two cells share is formed once:
+// lanes are columns (the east difference is minus the right lane's west
+// one, a face value goes to the downwind lane by shuffle) and the warp marches
+// along y from the upwind side (the difference to the row behind and the
+// face value on it are in registers).  Lanes at the ends and one row before
+// the first only feed the others: 29 of 32 lanes, 16 of 17 rows count (32 rows,
+// 8 warps per block: 582 us; 16 and 4: 565).  24 FP64 operations per cell and
+// ordinate, 4 more with the limiter and a division (140 cycles of the pipe)
+// where it acts; the cell-tile form before took FP64 comparisons, divisions
+// by the spacings and each shared quantity twice.  The same bits: the
+// limiter amplifies a rounding difference of 1e-16 to 3e-10 within 250
+// iterations.  256^2 S12, FP64: 748 -> 565 us, without the limiter 362 us.
+constexpr int kUwCols = 29, kUwRows = 16, kUwWarps = 4;
+static_assert(kUwRows <= 32, "one lane holds 1/dy of one row");
 
 template <typename T>
-__global__ void __launch_bounds__(256) uw2_residual_kernel(const Uw2Args<T> a)
+__global__ void __launch_bounds__(kUwWarps * 32) uw2_residual_kernel(const Uw2Args<T> a, int sx)
 {
-    __shared__ T sI[kLY][kLX];
-    __shared__ T sgx[kGY][kGX], sgy[kGY][kGX];
     if (a.done && ld_volatile_int(a.done)) return;
+    const int lane = threadIdx.x & 31, s = blockIdx.y * kUwWarps + (threadIdx.x >> 5);
+    if (s >= a.K) return;
     const int nx = a.nx, ny = a.ny, N = a.N, K = a.K;
-    const int i0 = blockIdx.x * kTX, j0 = blockIdx.y * kTY;
-    const int s0 = blockIdx.z * kDPB, s1 = min(K, s0 + kDPB);
-    const int tid = threadIdx.x;
-    // gradient-region cells of this thread (fixed across ordinates): weights in registers
-    constexpr int kG = (kGX * kGY + 255) / 256;
-    int gcell[kG];
-    T w4[kG][4], ghx[kG], ghy[kG];
-#pragma unroll
-    for (int u = 0; u < kG; ++u) {
-        const int q = tid + 256 * u;
-        gcell[u] = -1;
-        if (q < kGX * kGY) {
-            const int gr = q / kGX, gc = q - gr * kGX;
-            const int i = i0 - 1 + gc, j = j0 - 1 + gr;
-            if (i >= 0 && i < nx && j >= 0 && j < ny) {
-                const int c = i + nx * j;
-                gcell[u] = q;
-                w4[u][0] = a.gw[c];
-                w4[u][1] = a.gw[N + c];
-                w4[u][2] = a.gw[2 * (size_t)N + c];
-                w4[u][3] = a.gw[3 * (size_t)N + c];
-                ghx[u] = (T)a.dx[i];
-                ghy[u] = (T)a.dy[j];
-            }
+    const int bx = blockIdx.x % sx, by = blockIdx.x / sx;
+    const double mu = a.qmu[s], eta = a.qeta[s];
+    const bool xp = mu >= 0.0, yp = eta >= 0.0;
+    const int k = a.perm[s];
+    const int i = bx * kUwCols + lane - (xp ? 2 : 1);
+    const bool in = i >= 0 && i < nx;
+    const bool hE = in && i + 1 < nx, hW = in && i > 0;
+    const bool counts = in && (xp ? lane >= 2 && lane <= 30 : lane >= 1 && lane <= 29);
+    const int ic = min(max(i, 0), nx - 1);
+    const T hx = (T)a.dx[ic], hx2 = T(0.5) * hx, yx = T(1) / hx;
+    const T sx2 = xp ? hx2 : -hx2, am = (T)fabs(mu), ae = (T)fabs(eta);
+    const int ja = by * kUwRows, n = min(ny, ja + kUwRows) - ja;
+    const int dj = yp ? 1 : -1;
+    const int jf = yp ? ja : ja + n - 1;             // first row that counts
+    const T* Is = a.I + (size_t)s * N;
+    T* Rs = a.R + (size_t)s * N;
+    auto row_in = [&](int j) { return j >= 0 && j < ny; };
+    auto at = [&](int j) -> T {
+        if (!in || !row_in(j)) return T(0);
+        return value(a, Is, i + nx * j);
+    };
+    const int t0 = row_in(jf - dj) ? -1 : 0;
+    int j = jf + t0 * dj;
+    T Ic = at(j), vA = at(j + dj);
+    T dBn = row_in(j - dj) ? Ic - at(j - dj) : T(0);  // from the row behind
+    T fB = T(0);                                      // face value on its side
+    if (t0 == 0 && a.inflow && in) fB = (T)a.inflow[(size_t)(yp ? 2 * ny + i : 2 * ny + nx + i) * K + k];
+    // lane l: dy / 2 and 1/dy of row t = l
+    const T hl = (T)a.dy[min(max(jf + lane * dj, 0), ny - 1)], hl2 = T(0.5) * hl, ry = T(1) / hl;
+    const T hy2_up = t0 < 0 ? T(0.5) * (T)a.dy[jf - dj] : T(0);   // of the row before the first
+    for (int t = t0; t < n; ++t, j += dj) {
+        const int c = ic + nx * j;
+        const T vAA = at(j + 2 * dj);   // used in the next turn
+        const T wE = a.gw[c], wW = a.gw[N + c], wN = a.gw[2 * (size_t)N + c], wS = a.gw[3 * (size_t)N + c];
+        const T sv = a.src[c], sg = a.sigt[c];
+        T dE = __shfl_down_sync(kFull, Ic, 1) - Ic, dWn = __shfl_up_sync(kFull, dE, 1);
+        if (!hE) dE = T(0);   // a missing neighbour has weight 0 and difference 0
+        if (!hW) dWn = T(0);
+        const T dA = row_in(j + dj) ? vA - Ic : T(0);
+        T gx = fma(wW, -dWn, fma(wE, dE, T(0)));
+        T gy;
+        if (yp) gy = fma(wS, -dBn, fma(wN, dA, T(0)));
+        else gy = fma(wS, dA, fma(wN, -dBn, T(0)));
+        const T hs = __shfl_sync(kFull, hl2, t < 0 ? 0 : t), hy2 = t < 0 ? hy2_up : hs;
+        T psi;
+        if (a.limiter == 0 && limit(dE, dWn, dA, dBn, hx2 * gx, hy2 * gy, psi)) {
+            gx *= psi;
+            gy *= psi;
         }
-    }
-    // this thread's tile cell
-    const int tx = tid % kTX, ty = tid / kTX;
-    const int ic = i0 + tx, jc = j0 + ty;
-    const bool mine = ic < nx && jc < ny;
-    const int cc = mine ? ic + nx * jc : 0;
-    T srcc = T(0), sigc = T(0), hxc = T(1), hyc = T(1), hxW = T(1), hxE = T(1), hyS = T(1), hyN = T(1);
-    if (mine) {
-        srcc = a.src[cc];
-        sigc = a.sigt[cc];
-        hxc = (T)a.dx[ic];
-        hyc = (T)a.dy[jc];
-        if (ic > 0) hxW = (T)a.dx[ic - 1];
-        if (ic + 1 < nx) hxE = (T)a.dx[ic + 1];
-        if (jc > 0) hyS = (T)a.dy[jc - 1];
-        if (jc + 1 < ny) hyN = (T)a.dy[jc + 1];
-    }
-    for (int s = s0; s < s1; ++s) {
-        const T* Is = a.I + (size_t)s * N;
-        for (int q = tid; q < kLX * kLY; q += 256) {
-            const int r = q / kLX, c = q - r * kLX;
-            const int i = i0 - 2 + c, j = j0 - 2 + r;
-            T v = T(0);
-            if (i >= 0 && i < nx && j >= 0 && j < ny) v = value(a, Is, i + nx * j);
-            sI[r][c] = v;
+        const T fx = fma(sx2, gx, Ic);   // downwind faces
+        T fy;
+        if (yp) fy = fma(hy2, gy, Ic);
+        else fy = fma(-hy2, gy, Ic);
+        T fu = xp ? __shfl_up_sync(kFull, fx, 1) : __shfl_down_sync(kFull, fx, 1);
+        if (t >= 0) {
+            if (in && (xp ? i == 0 : i == nx - 1))
+                fu = a.inflow ? (T)a.inflow[(size_t)(xp ? j : ny + j) * K + k] : T(0);
+            // mu (E - W) = |mu| (downwind - upwind), the same bits
+            T r = fma(-sg, Ic, sv);
+            r -= div_by(am * (fx - fu), hx, yx);
+            r -= div_by(ae * (fy - fB), __shfl_sync(kFull, hl, t), __shfl_sync(kFull, ry, t));
+            if (counts) Rs[c] = r;
         }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < kG; ++u) {
-            if (gcell[u] < 0) continue;
-            const int q = gcell[u];
-            const int gr = q / kGX, gc = q - gr * kGX;
-            const int i = i0 - 1 + gc, j = j0 - 1 + gr;
-            const int r = gr + 1, c = gc + 1;   // position in sI
-            T gx, gy;
-            limited_gradient_vals(sI[r][c], i + 1 < nx, sI[r][c + 1], i > 0, sI[r][c - 1], j + 1 < ny, sI[r + 1][c],
-                                  j > 0, sI[r - 1][c], w4[u][0], w4[u][1], w4[u][2], w4[u][3], ghx[u], ghy[u],
-                                  a.limiter, gx, gy);
-            sgx[gr][gc] = gx;
-            sgy[gr][gc] = gy;
-        }
-        __syncthreads();
-        if (mine) {
-            const double mu = a.qmu[s], eta = a.qeta[s];
-            const int k = a.perm[s];
-            const int gr = ty + 1, gc = tx + 1, r = ty + 2, c = tx + 2;
-            const T Ic = sI[r][c], gx = sgx[gr][gc], gy = sgy[gr][gc];
-            T fE, fW, fN, fS;
-            if (mu >= 0.0) {
-                fE = fma(T(0.5) * hxc, gx, Ic);
-                fW = ic > 0 ? fma(T(0.5) * hxW, sgx[gr][gc - 1], sI[r][c - 1])
-                            : (a.inflow ? (T)a.inflow[(size_t)jc * K + k] : T(0));
-            } else {
-                fW = fma(T(-0.5) * hxc, gx, Ic);
-                fE = ic + 1 < nx ? fma(T(-0.5) * hxE, sgx[gr][gc + 1], sI[r][c + 1])
-                                 : (a.inflow ? (T)a.inflow[(size_t)(ny + jc) * K + k] : T(0));
-            }
-            if (eta >= 0.0) {
-                fN = fma(T(0.5) * hyc, gy, Ic);
-                fS = jc > 0 ? fma(T(0.5) * hyS, sgy[gr - 1][gc], sI[r - 1][c])
-                            : (a.inflow ? (T)a.inflow[(size_t)(2 * ny + ic) * K + k] : T(0));
-            } else {
-                fS = fma(T(-0.5) * hyc, gy, Ic);
-                fN = jc + 1 < ny ? fma(T(-0.5) * hyN, sgy[gr + 1][gc], sI[r + 1][c])
-                                 : (a.inflow ? (T)a.inflow[(size_t)(2 * ny + nx + ic) * K + k] : T(0));
-            }
-            T rr = srcc - sigc * Ic;
-            rr -= (T)mu * (fE - fW) / hxc;
-            rr -= (T)eta * (fN - fS) / hyc;
-            a.R[(size_t)s * N + cc] = rr;
-        }
-        __syncthreads();
+        fB = fy;
+        dBn = dA;
+        Ic = vA;
+        vA = vAA;
     }
 }
 
@@ -276,9 +295,10 @@ Uw2Args<T> uw2_args(const Plan& P, bool with_corr, const int* done)
 
 cudaError_t launch_uw2_residual(const Plan& P, cudaStream_t st)
 {
-    const dim3 grid((P.nx + kTX - 1) / kTX, (P.ny + kTY - 1) / kTY, (P.K + kDPB - 1) / kDPB);
-    if (P.fp32) uw2_residual_kernel<float><<<grid, 256, 0, st>>>(uw2_args<float>(P, true, &P.status->done));
-    else uw2_residual_kernel<double><<<grid, 256, 0, st>>>(uw2_args<double>(P, true, &P.status->done));
+    const int sx = (P.nx + kUwCols - 1) / kUwCols, sy = (P.ny + kUwRows - 1) / kUwRows;
+    const dim3 grid(sx * sy, (P.K + kUwWarps - 1) / kUwWarps);
+    if (P.fp32) uw2_residual_kernel<float><<<grid, kUwWarps * 32, 0, st>>>(uw2_args<float>(P, true, &P.status->done), sx);
+    else uw2_residual_kernel<double><<<grid, kUwWarps * 32, 0, st>>>(uw2_args<double>(P, true, &P.status->done), sx);
     return cudaGetLastError();
 }
 
