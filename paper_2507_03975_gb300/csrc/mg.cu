@@ -1541,13 +1541,19 @@ __global__ void __launch_bounds__(kTileBlock) mg_tile_grid_kernel(const TileArgs
 // are cut into row strips, one per CTA; the cut is made on level P = ld + 1
 // and doubled downwards, so a coarse cell and its children always live in
 // the same CTA and the grid transfers stay local.  Each strip array carries
-// one halo row above and below; a phase that writes a boundary row also
-// stores it into the neighbour's halo row (distributed shared memory) before
-// the cluster barrier, so every read after the barrier is local.  Levels P..
-// live whole in CTA 0: the other CTAs store their restricted rows of level P
-// into CTA 0, and CTA 0 stores level P's correction back into every CTA.
-// Reductions store each CTA's partial into every CTA's slot table and sum
-// the table in a fixed order: all CTAs get the same bits.
+// one halo row above and below; a pass that writes a boundary row also sends
+// it into the neighbour's halo row (distributed shared memory), and the pass
+// after it waits for the neighbours' rows, so every read is local.  Levels P..
+// live whole in CTA 0: the other CTAs send their restricted rows of level P
+// to CTA 0, and CTA 0 sends each CTA the rows of level P's correction over its
+// strip.  Reductions send each CTA's partial into every CTA's slot table and
+// sum the table in a fixed order: all CTAs get the same bits.
+//
+// Bound by the latency of its ~25 dependent passes and exchanges per inner
+// iteration (16 of 152 SMs; DRAM and arithmetic idle).  Per call, before and
+// after the sends, CTA 0's small_cycle, 512 threads and the asynchronous
+// coefficient copies: 64^2 to 1e-12 213 -> 115 us, 200^2 143 -> 103 us, 256^2 with
+// two inner iterations 79 -> 55 us.  The same bits.
 constexpr int kSA_D = 0, kSA_ID = 1, kSA_CX = 2, kSA_CY = 3, kSA_X = 4, kSA_T = 5, kSA_R = 6;
 constexpr int kSA_P = 7, kSA_DL = 8;   // level 0 only
 constexpr int kMaxCl = 16;
@@ -1572,15 +1578,17 @@ struct SArgs {
     const float* r0;       // b - D guess (FP32), computed with b
     const double* norms;   // [0] = |b - D guess|^2, [1] = |b|^2 (FP64)
     double rtol;
-    int max_iter, nu;
+    int max_iter;
     float inner_rtol, omega, alpha;
     Status* status;
+    long long wait_cycles;   // bound of the cluster barrier's wait
 };
 
 // This CTA's part of one level: rows [rs, rs + rows); array k at float
 // offset off + k * cap, cell (jj, i) at (jj + 1) * nx + i.
 struct Strip {
     int nx, ny, rs, rows, cap, off, prev_rows;
+    unsigned inv;      // 2^21 / nx, rounded up
     bool prev, next;   // neighbouring strips exist (strip levels only)
 };
 
@@ -1591,7 +1599,7 @@ __device__ __forceinline__ float* sarr(const Strip S, int k) { return sm_f + S.o
 __device__ __forceinline__ void strip_rows(const SArgs& a, int l, int r, int& rs, int& re)
 {
     const int P = a.ld + 1, nyP = a.lv[P].ny;
-    const int s0 = (int)((long long)r * nyP / a.cl), s1 = (int)((long long)(r + 1) * nyP / a.cl);
+    const int s0 = r * nyP / a.cl, s1 = (r + 1) * nyP / a.cl;   // below 2^25
     const int sh = P - l;
     rs = s0 << sh;
     re = min(s1 << sh, a.lv[l].ny);
@@ -1652,83 +1660,391 @@ __device__ __forceinline__ float strip_Av(const Strip S, int k, int c)
     return y;
 }
 
+// Threads of a strip CTA.  Every reduction is over 1024 virtual threads (virtual
+// thread v takes cells v, v + 1024, ...; this thread is v = threadIdx.x and v +
+// 512), so the sums do not depend on this number.  512: barriers of half the
+// warps, and the 4096 cells per CTA of a large plan keep them busy (256^2, two
+// inner iterations, with cluster barriers: 1024 threads 79.6 us a call, 512
+// 74.9, 256 86.7).
+constexpr int kStripBlock = 512;
+constexpr int kVirtual = 2;
+
+// Communication of the cluster's CTAs.  Values that another CTA needs go to it
+// with st.async, which counts their bytes on an mbarrier of the receiver when
+// they have arrived; the receiver waits for the bytes it expects.  No fence
+// and no cluster barrier is involved: an arrival that releases earlier remote
+// stores (barrier.cluster, or mbarrier.arrive.release.cluster after a block
+// barrier) took 1.0-1.7 thousand cycles here, and a V-cycle of the 64^2 mesh
+// has fourteen.
+//
+// Three kinds of exchange, each with its own barriers:
+//   halo       a pass's boundary rows, between neighbouring strips;
+//   sum        every CTA's partial sums, all to all;
+//   transfer   level P's residual to CTA 0, its correction back.
+// A neighbour may be one exchange ahead (it has this CTA's data, this CTA
+// still waits for its other neighbour's), so halo and sum alternate between
+// two barriers; it cannot be two ahead.  Transfers strictly take turns.  A
+// halo value is overwritten by a later pass of the neighbour only after this
+// CTA has sent it something computed after its last use: a boundary cell reads
+// only the halo cell beside it, and each array's next write is at least one
+// exchange later.
 class SCluster {
   public:
-    __device__ SCluster() : cl_(cg::this_cluster())
+    static constexpr int kBars = 5;   // halo[2], sum[2], transfer
+    __device__ SCluster(unsigned long long* bars, long long limit, int* err)
+        : cl_(cg::this_cluster()), bars_(smem_addr(bars)), limit_(limit), err_(err), halo_(0), sum_(0), xfer_(0)
     {
         rank_ = (int)cl_.block_rank();
         n_ = (int)cl_.num_blocks();
+        if (threadIdx.x < kBars) mbar_init(bars + threadIdx.x, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        cl_.sync();   // the barriers of every CTA are initialised
     }
-    __device__ void sync() { cl_.sync(); }
+    __device__ void sync() { cl_.sync(); }   // with global memory; also: no CTA leaves while another may store into it
     __device__ int rank() const { return rank_; }
     __device__ int size() const { return n_; }
-    template <typename V>
-    __device__ V* remote(V* p, int r) { return cl_.map_shared_rank(p, r); }
-    // Fixed-order sums over the cluster, identical bits in every thread of
-    // every CTA.  slots: [3][kMaxCl][2] rotating tables (a table is written
-    // again only after two more barriers, so one barrier per sum suffices).
-    template <typename V>
-    __device__ void sum2(V a, V b, V out[2], V* slots, int& rot, V* wsm)
+    // address in CTA q's shared memory of this CTA's shared address `a`
+    __device__ static unsigned at(unsigned a, int q)
     {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(kFull, a, o);
-            b += __shfl_xor_sync(kFull, b, o);
-        }
-        __syncthreads();   // wsm free (previous use complete)
-        if (lane == 0) {
-            wsm[wid] = a;
-            wsm[32 + wid] = b;
+        unsigned ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(q));
+        return ra;
+    }
+    // barrier (in CTA q) of the halo exchange that the current pass belongs to, and of the transfer
+    __device__ unsigned halo_bar(int q) const { return at(bars_ + 8u * (halo_ & 1u), q); }
+    __device__ unsigned xfer_bar(int q) const { return at(bars_ + 32u, q); }
+    __device__ static void send(unsigned addr, float v, unsigned bar)
+    {
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr),
+                     "r"(__float_as_uint(v)), "r"(bar)
+                     : "memory");
+    }
+    // End of a pass that sent halo rows: `bytes` from the neighbours have
+    // arrived, and the block's own accesses are ordered (block barrier).
+    __device__ bool halo_wait(unsigned bytes)
+    {
+        const unsigned k = halo_++;
+        return wait(bars_ + 8u * (k & 1u), bytes, (k >> 1) & 1u);
+    }
+    __device__ bool xfer_wait(unsigned bytes)
+    {
+        const unsigned k = xfer_++;
+        return wait(bars_ + 32u, bytes, k & 1u);
+    }
+    // Fixed-order sums over the cluster, identical bits in every thread of
+    // every CTA; also a block barrier.  slots: [2][kMaxCl][2], wsm: [64].
+    // TWO = false: only a, out[0].
+    template <bool TWO>
+    __device__ bool sum2(const float a[kVirtual], const float b[kVirtual], float out[2], float* slots, float* ws)
+    {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+        for (int u = 0; u < kVirtual; ++u) {
+            float x = a[u], y = b[u];
+            for (int o = 16; o > 0; o >>= 1) {
+                x += __shfl_xor_sync(kFull, x, o);
+                if (TWO) y += __shfl_xor_sync(kFull, y, o);
+            }
+            if (lane == 0) {
+                ws[u * (kStripBlock / 32) + wid] = x;
+                if (TWO) ws[32 + u * (kStripBlock / 32) + wid] = y;
+            }
         }
         __syncthreads();
-        V* table = slots + rot * (2 * kMaxCl);
+        const unsigned k = sum_++;
+        float* table = slots + (k & 1u) * (2 * kMaxCl);
+        const unsigned bar = bars_ + 16u + 8u * (k & 1u);
         if (threadIdx.x < n_) {   // thread q stores this CTA's partial into CTA q's table
-            V ta = V(0), tb = V(0);
-            for (int w = 0; w < nw; ++w) {
-                ta += wsm[w];
-                tb += wsm[32 + w];
+            float ta = 0.f, tb = 0.f;
+#pragma unroll
+            for (int w = 0; w < 32; ++w) {
+                ta += ws[w];
+                if (TWO) tb += ws[32 + w];
             }
-            V* dst = cl_.map_shared_rank(table, (int)threadIdx.x);
-            dst[2 * rank_] = ta;
-            dst[2 * rank_ + 1] = tb;
+            const int q = (int)threadIdx.x;
+            const unsigned dst = at(smem_addr(table + 2 * rank_), q), rb = at(bar, q);
+            send(dst, ta, rb);
+            if (TWO) send(dst + 4u, tb, rb);
         }
-        cl_.sync();
-        V s0 = lane < n_ ? table[2 * lane] : V(0), s1 = lane < n_ ? table[2 * lane + 1] : V(0);
-        for (int o = 16; o > 0; o >>= 1) {
+        if (!wait(bar, (TWO ? 8u : 4u) * (unsigned)n_, (k >> 1) & 1u)) return false;
+        // both halves of the warp hold the table of at most 16 entries
+        const int e = lane & (kMaxCl - 1);
+        float s0 = e < n_ ? table[2 * e] : 0.f, s1 = TWO && e < n_ ? table[2 * e + 1] : 0.f;
+        for (int o = kMaxCl / 2; o > 0; o >>= 1) {
             s0 += __shfl_xor_sync(kFull, s0, o);
-            s1 += __shfl_xor_sync(kFull, s1, o);
+            if (TWO) s1 += __shfl_xor_sync(kFull, s1, o);
         }
         out[0] = s0;
         out[1] = s1;
-        rot = (rot + 1) % 3;
+        return true;
+    }
+    // The sum of one double (the FP64 residual norm): a tree over the warps
+    // instead of a chain of FP64 additions of 64 cycles each.  slots: [2][kMaxCl].
+    __device__ bool sumd(double a, double& out, double* slots, double* ws)
+    {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kStripBlock / 32;
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kFull, a, o);
+        if (lane == 0) ws[wid] = a;
+        __syncthreads();
+        const unsigned k = sum_++;
+        double* table = slots + (k & 1u) * kMaxCl;
+        const unsigned bar = bars_ + 16u + 8u * (k & 1u);
+        if (threadIdx.x < 32) {
+            double t = lane < nw ? ws[lane] : 0.0;
+            for (int o = nw / 2; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+            t = __shfl_sync(kFull, t, 0);
+            if (lane < n_)
+                asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
+                                 at(smem_addr(table + rank_), lane)),
+                             "l"(__double_as_longlong(t)), "r"(at(bar, lane))
+                             : "memory");
+        }
+        if (!wait(bar, 8u * (unsigned)n_, (k >> 1) & 1u)) return false;
+        double s0 = lane < n_ ? table[lane] : 0.0;
+        for (int o = kMaxCl / 2; o > 0; o >>= 1) s0 += __shfl_xor_sync(kFull, s0, o);
+        out = __shfl_sync(kFull, s0, 0);
+        return true;
     }
 
   private:
+    // Phase `parity` of the barrier at shared address bar complete with `bytes`
+    // received (warp 0 polls), then a block barrier; after a wait beyond the
+    // bound kErrTimeout is raised and false returned, in every thread.
+    __device__ bool wait(unsigned bar, unsigned bytes, unsigned parity)
+    {
+        bool ok = true;
+        if (threadIdx.x < 32) {
+            if (threadIdx.x == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+            __syncwarp();
+            const long long t0 = clock64();
+            for (;;) {
+                unsigned done;
+                asm volatile("{\n\t.reg .pred p;\n\t"
+                             "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                             "selp.u32 %0, 1, 0, p;\n\t}"
+                             : "=r"(done)
+                             : "r"(bar), "r"(parity)
+                             : "memory");
+                ok = done != 0;
+                if (ok || clock64() - t0 > limit_) break;
+            }
+            if (!ok && threadIdx.x == 0) atomicOr(err_, kErrTimeout);
+        }
+        return __syncthreads_and(ok);
+    }
     cg::cluster_group cl_;
+    unsigned bars_;
+    long long limit_;
+    int* err_;
+    unsigned halo_, sum_, xfer_;   // exchanges completed
     int rank_, n_;
 };
 
 __device__ __forceinline__ int other_buf(int k) { return k == kSA_X ? kSA_T : kSA_X; }
 
+// Barrier of the first `n` threads of the block (n a multiple of 32; all of
+// them call it, with the same id > 0): a warp barrier for one warp.
+__device__ __forceinline__ void part_sync(int id, int n)
+{
+    if (n <= 32) __syncwarp();
+    else asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// The V-cycle on the levels l0.. of at most kSmallCells cells, whole in CTA
+// 0's shared memory: input R of level l0, output T of level l0.  Same
+// operations per cell as the general passes, with the first Jacobi step
+// taken from r directly (x1 = omega r / d at the neighbours again) and the
+// prolongation inside the step after it: five passes per level instead of
+// eight, no integer division, a level is visited by the warps that hold
+// cells of it, and levels of at most 32 cells live in one warp's registers
+// and shuffles.  16^2 and below: 12-23 -> 4 thousand cycles per V-cycle.
+constexpr int kSmallCells = 1024;   // at most 6 levels above 32 cells: barrier ids 1..6
+__device__ __forceinline__ void small_cycle(const Strip* St, int l0, int nl, float om, float alpha)
+{
+    const int tid = threadIdx.x;
+    auto warps_for = [](int n) { return min(kStripBlock, (n + 31) & ~31); };
+    // division of c < 1024 by nx <= 1024: c nx < 2^21, so the scaled reciprocal
+    // is exact enough
+    auto split = [](int c, int nx, unsigned inv, int& i, int& j) {
+        j = (int)(((unsigned long long)c * inv) >> 21);
+        i = c - j * nx;
+    };
+    int lt = l0;   // first level of one warp
+    while (lt < nl - 1 && St[lt].rows * St[lt].nx > 32) ++lt;
+    for (int l = l0; l < lt; ++l) {
+        const Strip L = St[l], C = St[l + 1];
+        const int n = L.rows * L.nx, nt = warps_for(n);
+        if (tid >= nt) break;
+        const float* base = sm_f + L.off;
+        const float *D = base + kSA_D * L.cap, *ID = base + kSA_ID * L.cap, *CX = base + kSA_CX * L.cap,
+                    *CY = base + kSA_CY * L.cap, *R = base + kSA_R * L.cap;
+        float *X = sarr(L, kSA_X), *T = sarr(L, kSA_T), *CR = sarr(C, kSA_R);
+        const int nx = L.nx;
+        for (int q = tid; q < n; q += nt) {   // T = one Jacobi step from x1
+            const int c = q + nx;
+            auto x1 = [&](int k) { return __fmul_rn(__fmul_rn(om, R[k]), ID[k]); };
+            const float xc = x1(c);
+            float y = D[c] * xc;
+            y -= CX[c] * x1(c + 1);
+            y -= CX[c - 1] * x1(c - 1);
+            y -= CY[c] * x1(c + nx);
+            y -= CY[c - nx] * x1(c - nx);
+            T[c] = xc + om * (R[c] - y) * ID[c];
+        }
+        part_sync(1 + l - l0, nt);
+        for (int q = tid; q < n; q += nt) {   // X = the residual
+            const int c = q + nx;
+            X[c] = R[c] - strip_Av(L, kSA_T, c);
+        }
+        part_sync(1 + l - l0, nt);
+        const int cn = C.rows * C.nx, cnx = C.nx;
+        for (int q = tid; q < cn; q += nt) {
+            int I, J;
+            split(q, cnx, C.inv, I, J);
+            float sum = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = 2 * I + (k & 1), j = 2 * J + (k >> 1);
+                if (i < nx && j < L.rows) sum += X[(j + 1) * nx + i];
+            }
+            CR[q + cnx] = sum;
+        }
+        part_sync(1 + l - l0, nt);
+    }
+    if (tid < 32) {   // levels lt..: lane = cell
+        const int c = tid;
+        // (A v)(lane) of the level with coefficients d, e, w, n, s; lanes
+        // outside the level hold 0, couplings to missing neighbours are 0
+        auto av = [&](int nx, float d, float e, float w, float nn, float ss, float v) {
+            float y = d * v;
+            y -= e * __shfl_sync(kFull, v, (c + 1) & 31);
+            y -= w * __shfl_sync(kFull, v, (c + 31) & 31);
+            y -= nn * __shfl_sync(kFull, v, (c + nx) & 31);
+            y -= ss * __shfl_sync(kFull, v, (c + 64 - nx) & 31);
+            return y;
+        };
+        struct Coef { float d, id, e, w, n, s; };
+        auto coefs = [&](const Strip& L) {
+            Coef k{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (c < L.rows * L.nx) {
+                const float* base = sm_f + L.off;
+                const int p = c + L.nx;
+                k.d = base[kSA_D * L.cap + p];
+                k.id = base[kSA_ID * L.cap + p];
+                k.e = base[kSA_CX * L.cap + p];
+                k.w = base[kSA_CX * L.cap + p - 1];
+                k.n = base[kSA_CY * L.cap + p];
+                k.s = base[kSA_CY * L.cap + p - L.nx];
+            }
+            return k;
+        };
+        float rc = 0.f;   // r of the lane's cell on the current level
+        if (c < St[lt].rows * St[lt].nx) rc = sarr(St[lt], kSA_R)[c + St[lt].nx];
+        for (int l = lt; l < nl - 1; ++l) {
+            const Strip L = St[l], C = St[l + 1];
+            const int nx = L.nx, p = c + nx;
+            const Coef k = coefs(L);
+            const float x1 = __fmul_rn(__fmul_rn(om, rc), k.id);
+            const float y1 = av(nx, k.d, k.e, k.w, k.n, k.s, x1);
+            const float x2 = x1 + om * (rc - y1) * k.id;
+            const float y2 = av(nx, k.d, k.e, k.w, k.n, k.s, x2);
+            const float res = rc - y2;
+            if (c < L.rows * nx) {   // for the way up
+                sarr(L, kSA_R)[p] = rc;
+                sarr(L, kSA_T)[p] = x2;
+            }
+            int I, J;
+            split(c, C.nx, C.inv, I, J);
+            float sum = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = 2 * I + (q & 1), j = 2 * J + (q >> 1);
+                const float v = __shfl_sync(kFull, res, (j * nx + i) & 31);
+                if (i < nx && j < L.rows) sum += v;
+            }
+            rc = c < C.rows * C.nx ? sum : 0.f;
+        }
+        float t;   // the correction of the current level
+        {
+            const Coef k = coefs(St[nl - 1]);
+            t = rc * k.id;
+        }
+        for (int l = nl - 2; l >= lt; --l) {
+            const Strip L = St[l], C = St[l + 1];
+            const int nx = L.nx, p = c + nx;
+            const Coef k = coefs(L);
+            const bool in = c < L.rows * nx;
+            const float r = in ? sarr(L, kSA_R)[p] : 0.f, x = in ? sarr(L, kSA_T)[p] : 0.f;
+            int i, j;
+            split(c, nx, L.inv, i, j);
+            const float tc = __shfl_sync(kFull, t, ((j >> 1) * C.nx + (i >> 1)) & 31);
+            float v = in ? __fmaf_rn(alpha, tc, x) : 0.f;
+            for (int q = 0; q < 2; ++q) {
+                const float y = av(nx, k.d, k.e, k.w, k.n, k.s, v);
+                v = v + om * (r - y) * k.id;
+            }
+            t = v;
+        }
+        if (c < St[lt].rows * St[lt].nx) sarr(St[lt], kSA_T)[c + St[lt].nx] = t;
+        __syncwarp();
+    }
+    for (int l = lt - 1; l >= l0; --l) {
+        const Strip L = St[l], C = St[l + 1];
+        const int n = L.rows * L.nx, nt = warps_for(n);
+        if (tid >= nt) continue;
+        part_sync(1 + l - l0, nt);   // the coarse correction
+        const float* base = sm_f + L.off;
+        const float *D = base + kSA_D * L.cap, *ID = base + kSA_ID * L.cap, *CX = base + kSA_CX * L.cap,
+                    *CY = base + kSA_CY * L.cap, *R = base + kSA_R * L.cap;
+        float *X = sarr(L, kSA_X), *T = sarr(L, kSA_T);
+        const float* ct = sarr(C, kSA_T) + C.nx;
+        const int nx = L.nx, ny = L.rows, cnx = C.nx;
+        for (int q = tid; q < n; q += nt) {   // X = one Jacobi step from T + alpha P t_coarse
+            const int c = q + nx;
+            int i, j;
+            split(q, nx, L.inv, i, j);
+            // a missing neighbour has coupling 0; its parent index stays inside
+            auto y0 = [&](int k, int ii, int jj) {
+                return __fmaf_rn(alpha, ct[(min(max(jj, 0), ny - 1) >> 1) * cnx + (min(max(ii, 0), nx - 1) >> 1)], T[k]);
+            };
+            const float yc = y0(c, i, j);
+            float y = D[c] * yc;
+            y -= CX[c] * y0(c + 1, i + 1, j);
+            y -= CX[c - 1] * y0(c - 1, i - 1, j);
+            y -= CY[c] * y0(c + nx, i, j + 1);
+            y -= CY[c - nx] * y0(c - nx, i, j - 1);
+            X[c] = yc + om * (R[c] - y) * ID[c];
+        }
+        part_sync(1 + l - l0, nt);
+        for (int q = tid; q < n; q += nt) {
+            const int c = q + nx;
+            T[c] = X[c] + om * (R[c] - strip_Av(L, kSA_X, c)) * ID[c];
+        }
+    }
+    __syncthreads();
+}
+
 __device__ __forceinline__ void strip_body(const SArgs& a)
 {
-    __shared__ float slots_f[3 * 2 * kMaxCl];
-    __shared__ double slots_d[3 * 2 * kMaxCl];
+    __shared__ float slots_f[2 * 2 * kMaxCl];
+    __shared__ double slots_d[2 * kMaxCl];
     __shared__ float wsm_f[64];
-    __shared__ double wsm_d[64];
+    __shared__ double wsm_d[32];
     __shared__ Strip St[kMaxLevels];
-    SCluster cx;
+    __shared__ unsigned long long cl_bar[SCluster::kBars];
     if (ld_volatile_int(&a.status->done)) return;   // same value in every CTA
-    const int r = cx.rank(), ld = a.ld, P = ld + 1, nl = a.nl, nu = a.nu;
+    SCluster cx(cl_bar, a.wait_cycles, &a.status->error);
+    const int r = cx.rank(), ld = a.ld, P = ld + 1, nl = a.nl;
     const float om = a.omega, alpha = a.alpha;
-    const int down_buf = (nu % 2) ? kSA_X : kSA_T;   // pre-smoothed iterate; post-smoothed: kSA_T
-    float* prev_sm = r > 0 ? cx.remote(sm_f, r - 1) : nullptr;
-    float* next_sm = r + 1 < cx.size() ? cx.remote(sm_f, r + 1) : nullptr;
+    const unsigned prev_sm = cx.at(smem_addr(sm_f), max(r - 1, 0));
+    const unsigned next_sm = cx.at(smem_addr(sm_f), min(r + 1, cx.size() - 1));
 
     if (threadIdx.x < nl) {
         const int l = threadIdx.x;
         Strip S;
         S.nx = a.lv[l].nx;
+        S.inv = ((1u << 21) + (unsigned)S.nx - 1u) / (unsigned)S.nx;
         S.ny = a.lv[l].ny;
         S.cap = a.lv[l].cap;
         S.off = a.lv[l].off;
@@ -1754,198 +2070,161 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
     }
     // zero every array (halo rows on the domain boundary stay zero)
     {
-        const int tot = a.lv[nl - 1].off + 7 * a.lv[nl - 1].cap;
-        for (int c = threadIdx.x; c < tot; c += blockDim.x) sm_f[c] = 0.f;
+        const int tot = (a.lv[nl - 1].off + 7 * a.lv[nl - 1].cap) / 4;   // caps are multiples of 4
+        float4* z4 = reinterpret_cast<float4*>(sm_f);
+        for (int c = threadIdx.x; c < tot; c += blockDim.x) z4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    // coefficients of the levels this CTA holds (and the south coupling of
-    // row 0): one flat index over all of them, 4 items' loads in flight per thread
-    __shared__ int first[kMaxLevels + 1];
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int l = 0; l < nl; ++l) {
-            first[l] = acc;
-            if (l <= ld || r == 0) acc += St[l].rows * St[l].nx + (St[l].rs > 0 ? St[l].nx : 0);
+    // coefficients of the levels this CTA holds, and the south coupling of
+    // row 0: contiguous in the level's arrays and here, so asynchronous copies
+    // of 16 bytes where both sides allow it, all in flight together
+    for (int l = 0; l < nl; ++l) {
+        if (l > ld && r != 0) break;
+        const Strip S = St[l];
+        const SLevel& L = a.lv[l];
+        const int n = S.rows * S.nx, g0 = S.rs * S.nx;
+        float *D = sarr(S, kSA_D) + S.nx, *CX = sarr(S, kSA_CX) + S.nx, *CY = sarr(S, kSA_CY) + S.nx;
+        if ((n | g0 | S.nx) % 4 == 0) {
+            for (int c = 4 * threadIdx.x; c < n; c += 4 * blockDim.x) {
+                mg_cp_async16_cg(D + c, L.gd + g0 + c);
+                mg_cp_async16_cg(CX + c, L.gcx + g0 + c);
+                mg_cp_async16_cg(CY + c, L.gcy + g0 + c);
+            }
+        } else {
+            for (int c = threadIdx.x; c < n; c += blockDim.x) {
+                mg_cp_async4(D + c, L.gd + g0 + c);
+                mg_cp_async4(CX + c, L.gcx + g0 + c);
+                mg_cp_async4(CY + c, L.gcy + g0 + c);
+            }
         }
-        first[nl] = acc;
+        if (S.rs > 0)
+            for (int c = threadIdx.x; c < S.nx; c += blockDim.x) mg_cp_async4(CY - S.nx + c, L.gcy + g0 - S.nx + c);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    {
-        const int tot = first[nl];
-        constexpr int U = 4;
-        for (int e0 = threadIdx.x; e0 < tot; e0 += U * blockDim.x) {
-            float dv[U], xv[U], yv[U];
-            int lv[U], cc[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int e = e0 + u * blockDim.x;
-                lv[u] = -1;
-                if (e < tot) {
-                    int l = 0;
-                    while (first[l + 1] <= e) ++l;
-                    const Strip S = St[l];
-                    const SLevel& L = a.lv[l];
-                    const int c = e - first[l] - (S.rs > 0 ? S.nx : 0);   // c < 0: south halo row
-                    const int g = S.rs * S.nx + c;
-                    lv[u] = l;
-                    cc[u] = c;
-                    yv[u] = L.gcy[g];
-                    if (c >= 0) {
-                        dv[u] = L.gd[g];
-                        xv[u] = L.gcx[g];
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (lv[u] < 0) continue;
-                const Strip S = St[lv[u]];
-                const int c = cc[u] + S.nx;   // padded index
-                sarr(S, kSA_CY)[c] = yv[u];
-                if (cc[u] >= 0) {
-                    sarr(S, kSA_D)[c] = dv[u];
-                    sarr(S, kSA_ID)[c] = 1.f / dv[u];
-                    sarr(S, kSA_CX)[c] = xv[u];
-                }
-            }
-        }
+    for (int l = 0; l < nl; ++l) {
+        if (l > ld && r != 0) break;
+        const Strip S = St[l];
+        const float* D = sarr(S, kSA_D) + S.nx;
+        float* ID = sarr(S, kSA_ID) + S.nx;
+        for (int c = threadIdx.x; c < S.rows * S.nx; c += blockDim.x) ID[c] = 1.f / D[c];
     }
     __syncthreads();
 
     // store v into array k of strip S at padded index c, and into the
     // neighbours' halo rows when c lies in the first or last row
+    unsigned pbar = 0, nbar = 0;   // the neighbours' barriers of the current exchange
     auto put = [&](const Strip S, int k, int c, float v) {
         sarr(S, k)[c] = v;
-        if (S.prev && c < 2 * S.nx) prev_sm[S.off + k * S.cap + S.prev_rows * S.nx + c] = v;
-        if (S.next && c >= S.rows * S.nx) next_sm[S.off + k * S.cap + c - S.rows * S.nx] = v;
+        if (S.prev && c < 2 * S.nx) cx.send(prev_sm + 4u * (unsigned)(S.off + k * S.cap + S.prev_rows * S.nx + c), v, pbar);
+        if (S.next && c >= S.rows * S.nx) cx.send(next_sm + 4u * (unsigned)(S.off + k * S.cap + c - S.rows * S.nx), v, nbar);
     };
-    // `steps` damped-Jacobi steps from buffer cur; returns the buffer of the
-    // result.  mode 0: strip level, every thread, cluster barriers; 1: level
-    // held whole by CTA 0, every thread, block barriers; 2: the same with the
-    // lanes of warp 0 alone and warp barriers (small levels).
-    auto jacobi = [&](const Strip S, int cur, int steps, int mode) {
+    bool ok = true;
+    // a pass that puts halo rows of strip S: `begin` before it, `end` after
+    auto begin = [&] {
+        pbar = cx.halo_bar(max(r - 1, 0));
+        nbar = cx.halo_bar(min(r + 1, cx.size() - 1));
+    };
+    auto end = [&](const Strip S) {
+        ok = ok && cx.halo_wait(4u * (unsigned)S.nx * ((S.prev ? 1u : 0u) + (S.next ? 1u : 0u)));
+    };
+    // One damped-Jacobi step from buffer cur into the other; its halo rows go
+    // to the neighbours unless nothing reads them.
+    auto jacobi = [&](const Strip S, int cur, bool halo) {
         const float* rr = sarr(S, kSA_R);
         const float* id = sarr(S, kSA_ID);
-        const int tid = mode == 2 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-        const int nt = mode == 2 ? 32 : (int)blockDim.x;
-        for (int k = 0; k < steps; ++k) {
-            if (mode == 0) cx.sync();
-            else if (mode == 1) __syncthreads();
-            else __syncwarp();
-            const int oth = other_buf(cur), c0 = cur;
-            const float* src = sarr(S, cur);
-            each_c(S, [&](int c) { put(S, oth, c, src[c] + om * (rr[c] - strip_Av(S, c0, c)) * id[c]); }, tid, nt);
-            cur = oth;
-        }
-        return cur;
-    };
-    // residual of buffer cur summed over 2x2 children into coarse rows
-    // row0.. of the padded coarse array cr (coarse width cnx), thread tid of nt
-    auto restrict_to = [&](const Strip S, int cur, float* cr, int cnx, int row0, int tid, int nt) {
-        const float* rr = sarr(S, kSA_R);
-        const int crows = (S.rows + 1) / 2, nx = S.nx;
-        for (int cc = tid; cc < crows * cnx; cc += nt) {
-            const int JJ = cc / cnx, I = cc - JJ * cnx;
-            float sum = 0.f;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = 2 * I + (q & 1), jj = 2 * JJ + (q >> 1);
-                if (i < nx && jj < S.rows) {
-                    const int c = (jj + 1) * nx + i;
-                    sum += rr[c] - strip_Av(S, cur, c);
-                }
-            }
-            cr[(row0 + JJ + 1) * cnx + I] = sum;
+        const float* src = sarr(S, cur);
+        float* dst = sarr(S, other_buf(cur));
+        auto value = [&](int c) { return src[c] + om * (rr[c] - strip_Av(S, cur, c)) * id[c]; };
+        if (halo) {
+            begin();
+            each_c(S, [&](int c) { put(S, other_buf(cur), c, value(c)); }, threadIdx.x, blockDim.x);
+            end(S);
+        } else {
+            each_c(S, [&](int c) { dst[c] = value(c); }, threadIdx.x, blockDim.x);
+            __syncthreads();
         }
     };
 
-    // z = M^{-1} s: one V-cycle, input level-0 R, output level-0 T
+    // levels P.. whole in CTA 0: the passes above on levels of more than
+    // kSmallCells cells, small_cycle below
+    int wl = P;
+    while (wl < nl - 1 && St[wl].rows * St[wl].nx > kSmallCells) ++wl;
+
+    // z = M^{-1} s: one V-cycle (two damped-Jacobi steps before and after),
+    // input level-0 R, output level-0 T.  Down over the strips (and CTA 0's
+    // large levels), then up, one copy of either in the program: the kernel
+    // runs once per call, and its instructions come from L2 the first time.
     auto vcycle = [&]() {
-        for (int l = 0; l <= ld; ++l) {   // down over the strips
+        for (int l = 0; l < wl; ++l) {
+            const bool strips = l <= ld;
             const Strip S = St[l];
+            begin();
             {
                 const float* rr = sarr(S, kSA_R);
                 const float* id = sarr(S, kSA_ID);
                 each_c(S, [&](int c) { put(S, kSA_X, c, om * rr[c] * id[c]); }, threadIdx.x, blockDim.x);
             }
-            const int cur = jacobi(S, kSA_X, nu - 1, 0);
-            cx.sync();
+            if (strips) end(S);
+            else __syncthreads();
+            jacobi(S, kSA_X, strips);   // X -> T
+            // the residual of T summed over 2x2 children
             const Strip C = St[l + 1];
-            if (l < ld) {
-                restrict_to(S, cur, sarr(C, kSA_R), C.nx, 0, threadIdx.x, blockDim.x);
-                __syncthreads();
-            } else {   // level P rows go to CTA 0
-                restrict_to(S, cur, cx.remote(sarr(C, kSA_R), 0), C.nx, S.rs / 2, threadIdx.x, blockDim.x);
+            float* cr = sarr(C, kSA_R);
+            const bool away = l == ld && r != 0;   // level P's rows go to CTA 0
+            const int row0 = l == ld ? S.rs / 2 : 0;
+            const unsigned dst = cx.at(smem_addr(cr), 0), bar = cx.xfer_bar(0);
+            const float* rr = sarr(S, kSA_R);
+            const int crows = (S.rows + 1) / 2, fx = S.nx, cnx = C.nx;
+            for (int cc = threadIdx.x; cc < crows * cnx; cc += blockDim.x) {
+                const int JJ = cc / cnx, I = cc - JJ * cnx;
+                float sum = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int i = 2 * I + (q & 1), jj = 2 * JJ + (q >> 1);
+                    if (i < fx && jj < S.rows) {
+                        const int c = (jj + 1) * fx + i;
+                        sum += rr[c] - strip_Av(S, kSA_T, c);
+                    }
+                }
+                const int o = (row0 + JJ + 1) * cnx + I;
+                if (away) cx.send(dst + 4u * (unsigned)o, sum, bar);
+                else cr[o] = sum;
+            }
+            if (l < ld || !strips) __syncthreads();
+            else {
+                if (r != 0) break;
+                ok = ok && cx.xfer_wait(4u * (unsigned)(C.nx * (C.rows - crows)));   // the other CTAs' rows
             }
         }
-        cx.sync();
-        if (r == 0) {   // levels P.. whole in CTA 0: every thread on levels of more
-                        // than 64 cells, warp 0 alone below (cheaper barriers)
-            int wl = P;
-            while (wl < nl - 1 && St[wl].rows * St[wl].nx > 64) ++wl;
-            auto down = [&](int l, int mode) {
-                const Strip L = St[l];
-                const int tid = mode == 2 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-                const int nt = mode == 2 ? 32 : (int)blockDim.x;
-                const float* rr = sarr(L, kSA_R);
-                const float* id = sarr(L, kSA_ID);
-                float* xv = sarr(L, kSA_X);
-                each_c(L, [&](int c) { xv[c] = om * rr[c] * id[c]; }, tid, nt);
-                const int cur = jacobi(L, kSA_X, nu - 1, mode);
-                if (mode == 2) __syncwarp();
-                else __syncthreads();
-                const Strip C = St[l + 1];
-                restrict_to(L, cur, sarr(C, kSA_R), C.nx, 0, tid, nt);
-                if (mode == 2) __syncwarp();
-                else __syncthreads();
-            };
-            auto up = [&](int l, int mode) {
-                const Strip L = St[l];
-                const Strip C = St[l + 1];
-                const int tid = mode == 2 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
-                const int nt = mode == 2 ? 32 : (int)blockDim.x;
-                float* xv = sarr(L, down_buf);
-                const float* ct = sarr(C, kSA_T);
-                each_cell(L, [&](int c, int i, int j) { xv[c] += alpha * ct[(j / 2 + 1) * C.nx + i / 2]; }, tid, nt);
-                jacobi(L, down_buf, nu, mode);
-                if (mode == 2) __syncwarp();
-                else __syncthreads();
-            };
-            for (int l = P; l < wl; ++l) down(l, 1);
-            if (threadIdx.x < 32) {
-                for (int l = wl; l < nl - 1; ++l) down(l, 2);
-                const Strip L = St[nl - 1];
-                const float* rr = sarr(L, kSA_R);
-                const float* id = sarr(L, kSA_ID);
-                float* tv = sarr(L, kSA_T);
-                each_c(L, [&](int c) { tv[c] = rr[c] * id[c]; }, (int)threadIdx.x, 32);
-                __syncwarp();
-                for (int l = nl - 2; l >= wl; --l) up(l, 2);
-            }
-            __syncthreads();
-            for (int l = wl - 1; l >= P; --l) up(l, 1);
-            __syncthreads();
-            // level P's correction into every other CTA
-            const Strip C = St[P];
-            const float* ct = sarr(C, kSA_T) + C.nx;
-            const int n = C.rows * C.nx;
-            for (int q = 1; q < cx.size(); ++q) {
-                float* dst = cx.remote(sarr(C, kSA_T), q) + C.nx;
-                for (int c = threadIdx.x; c < n; c += blockDim.x) dst[c] = ct[c];
-            }
-        }
-        cx.sync();
-        for (int l = ld; l >= 0; --l) {   // up over the strips
+        if (r == 0) small_cycle(St, wl, nl, om, alpha);
+        for (int l = wl - 1; l >= 0; --l) {
+            const bool strips = l <= ld;
+            if (!strips && r != 0) continue;
             const Strip S = St[l];
             const Strip C = St[l + 1];
-            const float* ct = sarr(C, kSA_T);
-            const float* xo = sarr(S, down_buf);
+            float* ct = sarr(C, kSA_T);
+            if (l == ld) {   // level P's correction: to every CTA the rows over its strip
+                if (r == 0) {
+                    for (int c = C.nx + threadIdx.x; c < (C.rows + 1) * C.nx; c += blockDim.x) {
+                        const int row = c / C.nx - 1;
+                        const int q = (int)(((long long)(row + 1) * cx.size() - 1) / C.ny);   // the strip cut there
+                        if (q > 0) cx.send(cx.at(smem_addr(ct + c), q), ct[c], cx.xfer_bar(q));
+                    }
+                } else {
+                    ok = ok && cx.xfer_wait(4u * (unsigned)(C.nx * ((S.rows + 1) / 2)));
+                }
+            }
+            float* xo = sarr(S, kSA_T);
             const int crow0 = l == ld ? S.rs / 2 : 0;   // level P is held whole
+            begin();
             each_cell(S, [&](int c, int i, int jj) {
-                put(S, down_buf, c, xo[c] + alpha * ct[(crow0 + jj / 2 + 1) * C.nx + i / 2]);
+                put(S, kSA_T, c, xo[c] + alpha * ct[(crow0 + jj / 2 + 1) * C.nx + i / 2]);
             });
-            jacobi(S, down_buf, nu, 0);
-            __syncthreads();
+            if (strips) end(S);
+            else __syncthreads();
+            jacobi(S, kSA_T, strips);
+            jacobi(S, kSA_X, false);
         }
     };
 
@@ -1956,21 +2235,29 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
     float* dl_ = sarr(S0, kSA_DL) + nx;
     const float* z_ = sarr(S0, kSA_T) + nx;
     const float* p_ = sarr(S0, kSA_P) + nx;
-    int rotf = 0, rotd = 0;
     int total = 0;
-    double relres = 0.0;
+    double rr = 0.0;
+    bool spent = false, bad = false;
     const double bb = a.norms[1];
-    __shared__ int stop_now;
+    const double stop2 = a.rtol * a.rtol * bb;
+    // this thread's cells (index within the strip) as those of its virtual threads
+    auto each_v = [&](auto f) {
+        for (int c = threadIdx.x; c < n0; c += kVirtual * kStripBlock) {
+#pragma unroll
+            for (int u = 0; u < kVirtual; ++u)
+                if (c + u * kStripBlock < n0) f(c + u * kStripBlock, u);
+        }
+    };
     for (int outer = 0;; ++outer) {
         // residual s = b - D x: from the right-hand-side pass on the first
         // pass (x = guess), else in FP64 here
-        double rr;
         if (outer == 0) {
             for (int c = threadIdx.x; c < n0; c += blockDim.x) {
                 s_[c] = a.r0[g00 + c];
                 dl_[c] = 0.f;
             }
             rr = a.norms[0];
+            __syncthreads();
         } else {
             cx.sync();   // every CTA's x update visible
             double lrr = 0.0;
@@ -2006,94 +2293,91 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
                     }
                 }
             }
-            double v2[2];
-            cx.sum2<double>(lrr, 0.0, v2, slots_d, rotd, wsm_d);
-            rr = v2[0];
+            if (!(ok = cx.sumd(lrr, rr, slots_d, wsm_d))) break;
         }
-        // stop test in one thread (FP64 is slow here; every thread reads the decision)
-        if (threadIdx.x == 0) {
-            relres = bb > 0.0 ? sqrt(rr / bb) : 0.0;
-            stop_now = (rr <= a.rtol * a.rtol * bb || total >= a.max_iter) ? 1 : 0;
-        }
-        __syncthreads();
-        if (stop_now) {
+        // every thread holds the same rr
+        if (rr <= stop2 || total >= a.max_iter) {
             if (outer == 0)
                 for (int c = threadIdx.x; c < n0; c += blockDim.x) a.x[g00 + c] = a.guess[g00 + c];
             break;
         }
         // FP32 MG-PCG for D d = s, d = 0 to start
-        vcycle();
-        float f2[2];
-        {
-            float l0 = 0.f, l1 = 0.f;
-            each_c(S0, [&](int c) {
-                const float z = z_[c - nx], sv = s_[c - nx];
-                put(S0, kSA_P, c, z);
-                l0 += sv * z;
-                l1 += sv * sv;
-            }, threadIdx.x, blockDim.x);
-            cx.sum2<float>(l0, l1, f2, slots_f, rotf, wsm_f);
-        }
-        float rz = f2[0];
-        if (!(rz > 0.f) || !(rz < INFINITY) || !isfinite(rr)) {
-            // as in mg_solve_body: no usable FP32 search direction, leave the
-            // refinement (every CTA holds the same rz and rr); a non-finite
-            // residual poisons x, a vanished one keeps the current x
-            const bool bad = !(rz == 0.f) || !isfinite(rr);
-            const double* xo = outer == 0 ? a.guess : a.x;
-            for (int c = threadIdx.x; c < n0; c += blockDim.x) a.x[g00 + c] = bad ? kNaN : xo[g00 + c];
-            if (bad) relres = kNaN;
-            break;
-        }
-        const float istop = a.inner_rtol * a.inner_rtol * f2[1];
-        while (total < a.max_iter && rz > 0.f) {
-            // the previous barrier published p and its halo rows
-            float lpq = 0.f;
-            each_c(S0, [&](int c) { lpq += p_[c - nx] * strip_Av(S0, kSA_P, c); }, threadIdx.x, blockDim.x);
-            cx.sum2<float>(lpq, 0.f, f2, slots_f, rotf, wsm_f);
-            const float al = rz / f2[0];
-            float lss = 0.f;
-            each_c(S0, [&](int c) {   // q = A p again (same bits) instead of storing it
-                dl_[c - nx] += al * p_[c - nx];
-                const float sc = s_[c - nx] - al * strip_Av(S0, kSA_P, c);
-                s_[c - nx] = sc;
-                lss += sc * sc;
-            }, threadIdx.x, blockDim.x);
-            ++total;
-            cx.sum2<float>(lss, 0.f, f2, slots_f, rotf, wsm_f);
-            if (f2[0] <= istop || total >= a.max_iter) break;
+        float rz = 0.f, istop = 0.f, f2[2];
+        bool leave = false;
+        for (bool first = true;; first = false) {
             vcycle();
-            float lrz = 0.f;
-            for (int c = threadIdx.x; c < n0; c += blockDim.x) lrz += s_[c] * z_[c];
-            cx.sum2<float>(lrz, 0.f, f2, slots_f, rotf, wsm_f);
-            const float be = f2[0] / rz;
-            rz = f2[0];
-            each_c(S0, [&](int c) { put(S0, kSA_P, c, z_[c - nx] + be * p_[c - nx]); }, threadIdx.x, blockDim.x);
-            cx.sync();   // p and its halo rows visible before the product
+            if (!ok) break;
+            if (first) {
+                float l0[kVirtual] = {}, l1[kVirtual] = {};
+                begin();
+                each_v([&](int c, int u) {
+                    const float z = z_[c], sv = s_[c];
+                    put(S0, kSA_P, c + nx, z);
+                    l0[u] += sv * z;
+                    l1[u] += sv * sv;
+                });
+                end(S0);   // p and its halo rows visible before the product
+                if (!(ok = ok && cx.sum2<true>(l0, l1, f2, slots_f, wsm_f))) break;
+                rz = f2[0];
+                if (!(rz > 0.f) || !(rz < INFINITY) || !isfinite(rr)) {
+                    // as in mg_solve_body: no usable FP32 search direction, leave the
+                    // refinement (every CTA holds the same rz and rr); a non-finite
+                    // residual poisons x, a vanished one keeps the current x
+                    bad = !(rz == 0.f) || !isfinite(rr);
+                    const double* xo = outer == 0 ? a.guess : a.x;
+                    for (int c = threadIdx.x; c < n0; c += blockDim.x) a.x[g00 + c] = bad ? kNaN : xo[g00 + c];
+                    leave = true;
+                    break;
+                }
+                istop = a.inner_rtol * a.inner_rtol * f2[1];
+            } else {
+                float lrz[kVirtual] = {}, no[kVirtual] = {};
+                each_v([&](int c, int u) { lrz[u] += s_[c] * z_[c]; });
+                if (!(ok = cx.sum2<false>(lrz, no, f2, slots_f, wsm_f))) break;
+                const float be = f2[0] / rz;
+                rz = f2[0];
+                begin();
+                each_c(S0, [&](int c) { put(S0, kSA_P, c, z_[c - nx] + be * p_[c - nx]); }, threadIdx.x, blockDim.x);
+                end(S0);
+                if (!ok) break;
+            }
+            if (!(total < a.max_iter && rz > 0.f)) break;
+            float lpq[kVirtual] = {}, lss[kVirtual] = {}, no[kVirtual] = {};
+            each_v([&](int c, int u) { lpq[u] += p_[c] * strip_Av(S0, kSA_P, c + nx); });
+            if (!(ok = cx.sum2<false>(lpq, no, f2, slots_f, wsm_f))) break;
+            const float al = rz / f2[0];
+            each_v([&](int c, int u) {   // q = A p again (same bits) instead of storing it
+                dl_[c] += al * p_[c];
+                const float sc = s_[c] - al * strip_Av(S0, kSA_P, c + nx);
+                s_[c] = sc;
+                lss[u] += sc * sc;
+            });
+            ++total;
+            if (!(ok = cx.sum2<false>(lss, no, f2, slots_f, wsm_f))) break;
+            if (f2[0] <= istop || total >= a.max_iter) break;
         }
+        if (!ok || leave) break;
         {
             const double* xo = outer == 0 ? a.guess : a.x;
             for (int c = threadIdx.x; c < n0; c += blockDim.x) a.x[g00 + c] = xo[g00 + c] + (double)dl_[c];
         }
         if (total >= a.max_iter) {   // budget spent: no further residual evaluation
-            relres = -1.0;
+            spent = true;
             break;
         }
-        __syncthreads();   // stop_now is rewritten by thread 0 on the next pass
     }
     if (r == 0 && threadIdx.x == 0) {
         a.status->synth_iters = total;
         a.status->synth_iters_total += total;
-        a.status->synth_relres = relres;
+        a.status->synth_relres = bad ? kNaN : spent ? -1.0 : bb > 0.0 ? sqrt(rr / bb) : 0.0;
     }
-    // no CTA may leave while another can still store into its shared memory
     cx.sync();
 }
 
-__global__ void __launch_bounds__(kMgBlock) mg_strip_kernel(const SArgs a) { strip_body(a); }
+__global__ void __launch_bounds__(kStripBlock) mg_strip_kernel(const SArgs a) { strip_body(a); }
 
 // One cluster per problem: cluster c solves the problem of tab[c].
-__global__ void __launch_bounds__(kMgBlock) mg_strip_batch_kernel(const SArgs* __restrict__ tab)
+__global__ void __launch_bounds__(kStripBlock) mg_strip_batch_kernel(const SArgs* __restrict__ tab)
 {
     strip_body(tab[blockIdx.x / cg::this_cluster().num_blocks()]);
 }
@@ -2134,46 +2418,57 @@ int mg_setup_launches(const Plan& P)
 namespace {
 
 // Strip plan for cluster size cl: false if level 1 has fewer rows than CTAs
-// or the levels do not fit the shared memory of one CTA.
+// or the levels do not fit the shared memory of one CTA.  The levels from P
+// on are held whole by CTA 0: of the cuts that fit, the first with at most
+// kSmallCells cells at level P.  A pass over a strip level costs an exchange
+// between the CTAs (about 1000 cycles with the pass), one inside CTA 0's
+// small_cycle 350-450 (64^2: P = 32^2 instead of 16^2).  The cut changes no
+// result: every level's arithmetic is the same in either place.
 bool strip_plan(const Plan& P, int cl, size_t smem_cap, SArgs& sa, size_t& bytes)
 {
     const MgPlan& g = P.mg;
     if (cl < 2 || cl > kMaxCl || g.nl < 2) return false;
-    int ld = -1;
+    int last = -1;   // deepest possible strip level: the next has a row for every CTA
     for (int l = 0; l + 1 < g.nl; ++l)
-        if (g.ny[l + 1] >= cl) ld = l;
-    if (ld < 0) return false;
-    const int Pl = ld + 1, nyP = g.ny[Pl];
-    size_t off = 0;
-    for (int l = 0; l < g.nl; ++l) {
-        int rows = g.ny[l];
-        if (l <= ld) {
-            rows = 0;
-            for (int r = 0; r < cl; ++r) {
-                const int s0 = (int)((long long)r * nyP / cl), s1 = (int)((long long)(r + 1) * nyP / cl);
-                const int rs = s0 << (Pl - l), re = std::min(s1 << (Pl - l), g.ny[l]);
-                rows = std::max(rows, re - rs);
+        if (g.ny[l + 1] >= cl) last = l;
+    if (last < 0) return false;
+    for (int ld = 0; ld <= last; ++ld) {
+        if (ld < last && (long long)g.nx[ld + 1] * g.ny[ld + 1] > kSmallCells) continue;
+        const int Pl = ld + 1, nyP = g.ny[Pl];
+        size_t off = 0;
+        bool fits = true;
+        for (int l = 0; l < g.nl && fits; ++l) {
+            int rows = g.ny[l];
+            if (l <= ld) {
+                rows = 0;
+                for (int r = 0; r < cl; ++r) {
+                    const int s0 = (int)((long long)r * nyP / cl), s1 = (int)((long long)(r + 1) * nyP / cl);
+                    const int rs = s0 << (Pl - l), re = std::min(s1 << (Pl - l), g.ny[l]);
+                    rows = std::max(rows, re - rs);
+                }
             }
+            long long cap = (long long)(rows + 2) * g.nx[l];
+            cap = (cap + 3) / 4 * 4;   // 16-byte aligned arrays
+            const int narr = l == 0 ? 9 : 7;
+            sa.lv[l] = SLevel{g.nx[l], g.ny[l], (int)cap, (int)off, g.d[l], g.cx[l], g.cy[l]};
+            off += (size_t)narr * (size_t)cap;
+            fits = off * sizeof(float) <= smem_cap;
         }
-        long long cap = (long long)(rows + 2) * g.nx[l];
-        cap = (cap + 3) / 4 * 4;   // 16-byte aligned arrays
-        const int narr = l == 0 ? 9 : 7;
-        sa.lv[l] = SLevel{g.nx[l], g.ny[l], (int)cap, (int)off, g.d[l], g.cx[l], g.cy[l]};
-        off += (size_t)narr * (size_t)cap;
-        if (off * sizeof(float) > smem_cap) return false;
+        if (!fits) continue;
+        sa.nl = g.nl;
+        sa.ld = ld;
+        sa.cl = cl;
+        bytes = off * sizeof(float);
+        return true;
     }
-    sa.nl = g.nl;
-    sa.ld = ld;
-    sa.cl = cl;
-    bytes = off * sizeof(float);
-    return true;
+    return false;
 }
 
 cudaError_t launch_cluster(const void* fn, void** args, int cl, size_t smem, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(kMgBlock);
+    cfg.blockDim = dim3(kStripBlock);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
@@ -2190,7 +2485,7 @@ int clusters_fit(const void* fn, int cl, size_t smem)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(kMgBlock);
+    cfg.blockDim = dim3(kStripBlock);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -2314,11 +2609,11 @@ void strip_fill(const Plan& P, const double* guess, double* out, SArgs& sa)
     sa.norms = P.partials + (size_t)4 * kMaxCgBlocks;
     sa.rtol = P.synth_rtol;
     sa.max_iter = P.synth_max_iter;
-    sa.nu = 2;
     sa.inner_rtol = 1e-4f;
     sa.omega = 0.8f;
     sa.alpha = 1.8f;
     sa.status = P.status;
+    sa.wait_cycles = P.wait_cycles;
 }
 
 MgArgs fallback_args(const Plan& P, const double* guess, double* out, size_t& smem)
@@ -2418,7 +2713,7 @@ cudaError_t launch_synthetic_solve(const Plan& P, const double* guess, double* o
     if (P.synth_cl > 0) {
         SArgs sa{};
         size_t bytes = 0;
-        if (!strip_plan(P, P.synth_cl, (size_t)-1, sa, bytes)) return cudaErrorInvalidConfiguration;
+        if (!strip_plan(P, P.synth_cl, strip_smem_cap(), sa, bytes)) return cudaErrorInvalidConfiguration;
         strip_fill(P, guess, out, sa);
         void* args[] = {&sa};
         return launch_cluster((const void*)mg_strip_kernel, args, P.synth_cl, bytes, st);
@@ -2484,7 +2779,7 @@ cudaError_t launch_strip_batch(const void* tab, int n, int cl, size_t bytes, cud
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(n * cl);
-    cfg.blockDim = dim3(kMgBlock);
+    cfg.blockDim = dim3(kStripBlock);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
