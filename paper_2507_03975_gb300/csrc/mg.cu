@@ -321,16 +321,18 @@ class GridCtx {
     __device__ void sync()
     {
         __syncthreads();
-        if (threadIdx.x == 0 && !ld_volatile_int(&a_.status->error)) {
+        if (threadIdx.x == 0 && !failed_) {
             const unsigned inc = blockIdx.x == 0 ? kFlip - (gridDim.x - 1u) : 1u;
             asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(a_.gbar), "r"(inc) : "memory");
             phase_ ^= kFlip;
             const long long t0 = clock64();
-            while ((ld_acquire_u32(a_.gbar) & kFlip) != phase_) {
-                if (clock64() - t0 > a_.wait_cycles) {
-                    atomicOr(&a_.status->error, kErrTimeout);
-                    break;
-                }
+            // another CTA's time-out ends the wait too; looked at every 64 polls
+            // (before every arrival it cost a round trip to L2 per barrier)
+            for (unsigned n = 1; (ld_acquire_u32(a_.gbar) & kFlip) != phase_; ++n) {
+                failed_ = clock64() - t0 > a_.wait_cycles;
+                if (failed_) atomicOr(&a_.status->error, kErrTimeout);
+                else if (n % 64 == 0) failed_ = ld_volatile_int(&a_.status->error) != 0;
+                if (failed_) break;
             }
         }
         __syncthreads();
@@ -341,48 +343,40 @@ class GridCtx {
         if (local) return Range{(int)threadIdx.x, (int)blockDim.x, blockIdx.x == 0};
         return Range{(int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x), true};
     }
-    __device__ void sum2f(float a, float b, float out[2], float*, int& rot)
-    {
-        a = blockf(a);
-        b = blockf(b);
-        float* tab = a_.gslots_f + (size_t)rot * 2 * gridDim.x;
-        if (threadIdx.x == 0) {
-            tab[2 * blockIdx.x] = a;
-            tab[2 * blockIdx.x + 1] = b;
-        }
-        sync();
-        float s0 = 0.f, s1 = 0.f;
-        table_sum(tab, s0, s1);
-        for (int o = 16; o > 0; o >>= 1) {
-            s0 += __shfl_xor_sync(kFull, s0, o);
-            s1 += __shfl_xor_sync(kFull, s1, o);
-        }
-        out[0] = s0;
-        out[1] = s1;
-        rot = (rot + 1) % 3;
-    }
-    __device__ void sum2d(double a, double b, double out[2], double*, int& rot)
-    {
-        a = blockd(a);
-        b = blockd(b);
-        double* tab = a_.gslots_d + (size_t)rot * 2 * gridDim.x;
-        if (threadIdx.x == 0) {
-            tab[2 * blockIdx.x] = a;
-            tab[2 * blockIdx.x + 1] = b;
-        }
-        sync();
-        double s0 = 0.0, s1 = 0.0;
-        table_sum(tab, s0, s1);
-        for (int o = 16; o > 0; o >>= 1) {
-            s0 += __shfl_xor_sync(kFull, s0, o);
-            s1 += __shfl_xor_sync(kFull, s1, o);
-        }
-        out[0] = s0;
-        out[1] = s1;
-        rot = (rot + 1) % 3;
-    }
+    // Fixed-order sums over the grid, the same bits everywhere; also a barrier.
+    // One warp per CTA reads the table: with all of them 2432 warps read the
+    // same few lines at once (8 thousand cycles per sum; 4.4 now).
+    __device__ void sum2f(float a, float b, float out[2], float* res, int& rot) { sum2(a, b, out, res, a_.gslots_f, rot); }
+    __device__ void sum2d(double a, double b, double out[2], double* res, int& rot) { sum2(a, b, out, res, a_.gslots_d, rot); }
 
   private:
+    template <typename T>
+    __device__ void sum2(T a, T b, T out[2], T* res, T* slots, int& rot)
+    {
+        block2(a, b);
+        T* tab = slots + (size_t)rot * 2 * gridDim.x;
+        if (threadIdx.x == 0) {
+            tab[2 * blockIdx.x] = a;
+            tab[2 * blockIdx.x + 1] = b;
+        }
+        sync();
+        if (threadIdx.x < 32) {
+            T s0 = T(0), s1 = T(0);
+            table_sum(tab, s0, s1);
+            for (int o = 16; o > 0; o >>= 1) {
+                s0 += __shfl_xor_sync(kFull, s0, o);
+                s1 += __shfl_xor_sync(kFull, s1, o);
+            }
+            if (threadIdx.x == 0) {   // res: two slots, read before the next sum's barriers
+                res[0] = s0;
+                res[1] = s1;
+            }
+        }
+        __syncthreads();
+        out[0] = res[0];
+        out[1] = res[1];
+        rot = (rot + 1) % 3;
+    }
     static constexpr unsigned kFlip = 0x80000000u;
     __device__ static unsigned ld_acquire_u32(const unsigned* p)
     {
@@ -414,31 +408,32 @@ class GridCtx {
                 }
         }
     }
-    __device__ float blockf(float v)
+    // Both block sums in thread 0 (the same order as a butterfly over the warps).
+    template <typename T>
+    __device__ void block2(T& a, T& b)
     {
-        __shared__ float w[32];
+        __shared__ T w[64];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(kFull, a, o);
+            b += __shfl_xor_sync(kFull, b, o);
+        }
+        if (lane == 0) {   // its last readers have passed two barriers since
+            w[wid] = a;
+            w[32 + wid] = b;
+        }
         __syncthreads();
-        if (lane == 0) w[wid] = v;
-        __syncthreads();
-        float t = lane < nw ? w[lane] : 0.f;
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-        return t;
-    }
-    __device__ double blockd(double v)
-    {
-        __shared__ double w[32];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-        __syncthreads();
-        if (lane == 0) w[wid] = v;
-        __syncthreads();
-        double t = lane < nw ? w[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-        return t;
+        if (wid == 0) {
+            a = lane < nw ? w[lane] : T(0);
+            b = lane < nw ? w[32 + lane] : T(0);
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(kFull, a, o);
+                b += __shfl_xor_sync(kFull, b, o);
+            }
+        }
     }
     const MgArgs& a_;
+    bool failed_ = false;  // thread 0: a wait ran out (here or in another CTA)
     unsigned phase_ = 0;   // thread 0: the barrier word's top bit after the last completed barrier
 };
 
@@ -1022,8 +1017,15 @@ __device__ __forceinline__ void tile_load(TileView& v, float* base, int cells, c
 // loop can make the compiler reload them.
 struct LocalLevel {
     int nx, ny;
-    int d, cx, cy, id, x, t, r;
+    unsigned inv;                 // 2^32 / nx, rounded up (nx > 1)
+    int d, cx, cy, id, x, t, r;   // offsets of cell 0: a ghost row lies before and after every array
 };
+
+// Floats of one level: its arrays with their ghost rows, a multiple of 4.
+__host__ __device__ __forceinline__ int local_floats(int nx, int ny)
+{
+    return (kLocalArrays * nx * (ny + 2) + 3) & ~3;
+}
 
 // One array of a LocalLevel in the dynamic shared memory.
 struct LocalArr {
@@ -1041,40 +1043,55 @@ struct LocalView {
         : nx(L.nx), ny(L.ny), d{L.d}, cx{L.cx}, cy{L.cy}, id{L.id}, x{L.x}, t{L.t}, r{L.r} {}
 };
 
-__device__ __forceinline__ void local_down(const LocalLevel Ls, const LocalLevel Cs, float om)
+// Row of cell c (c nx < 2^32).
+__device__ __forceinline__ int local_row(const LocalLevel& L, int c)
+{
+    return L.nx > 1 ? (int)__umulhi((unsigned)c, L.inv) : c;
+}
+
+// Threads that visit a level of n cells, and the barrier among them (level
+// ids 1..7: at most seven levels between 4096 and kDirectMax cells).
+__device__ __forceinline__ int local_threads(int n) { return min(kTileBlock, (n + 31) & ~31); }
+__device__ __forceinline__ void local_sync(int id, int nt)
+{
+    if (nt <= 32) __syncwarp();
+    else asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(nt) : "memory");
+}
+
+// The passes are branch-free: a coupling to a missing neighbour is 0 (the
+// operators have zero face coefficients on the domain's edge, ghost rows are
+// zeroed once), every neighbour index stays inside the padded arrays, and no
+// thread divides.  The fused multiply-adds of the last sums are written out:
+// which of two products is fused is otherwise the compiler's choice.
+__device__ __forceinline__ void local_down(const LocalLevel Ls, const LocalLevel Cs, float om, int id)
 {
     const LocalView L(Ls), C(Cs);
-    const int tid = threadIdx.x, nt = blockDim.x;
-    auto sync = [] { __syncthreads(); };
-    const int nx = L.nx, ny = L.ny, n = nx * ny;
+    const int nx = L.nx, ny = L.ny, n = nx * ny, nt = local_threads(n), tid = threadIdx.x;
+    if (tid >= nt) return;
     auto x1 = [&](int c) { return om * L.r[c] * L.id[c]; };
-    int i = tid % nx, j = tid / nx;
-    const int di = nt % nx, dj = nt / nx;
-    auto step = [&] { i += di; j += dj; if (i >= nx) { i -= nx; ++j; } };
-    for (int c = tid; c < n; c += nt, step()) {
+#pragma unroll 2
+    for (int c = tid; c < n; c += nt) {
         float nb = L.r[c];
-        if (i + 1 < nx) nb += L.cx[c] * x1(c + 1);
-        if (i > 0) nb += L.cx[c - 1] * x1(c - 1);
-        if (j + 1 < ny) nb += L.cy[c] * x1(c + nx);
-        if (j > 0) nb += L.cy[c - nx] * x1(c - nx);
-        L.x[c] = (1.f - om) * x1(c) + om * nb * L.id[c];
+        nb += L.cx[c] * x1(c + 1);
+        nb += L.cx[c - 1] * x1(c - 1);
+        nb += L.cy[c] * x1(c + nx);
+        nb += L.cy[c - nx] * x1(c - nx);
+        L.x[c] = __fmaf_rn(om * nb, L.id[c], __fmul_rn(1.f - om, x1(c)));
     }
-    sync();
-    i = tid % nx;
-    j = tid / nx;
-    for (int c = tid; c < n; c += nt, step()) {
+    local_sync(id, nt);
+#pragma unroll 2
+    for (int c = tid; c < n; c += nt) {
         float res = L.r[c] - L.d[c] * L.x[c];
-        if (i + 1 < nx) res += L.cx[c] * L.x[c + 1];
-        if (i > 0) res += L.cx[c - 1] * L.x[c - 1];
-        if (j + 1 < ny) res += L.cy[c] * L.x[c + nx];
-        if (j > 0) res += L.cy[c - nx] * L.x[c - nx];
+        res += L.cx[c] * L.x[c + 1];
+        res += L.cx[c - 1] * L.x[c - 1];
+        res += L.cy[c] * L.x[c + nx];
+        res += L.cy[c - nx] * L.x[c - nx];
         L.t[c] = res;
     }
-    sync();
+    local_sync(id, nt);
     const int cnx = C.nx, cn = cnx * C.ny;
-    int I = tid % cnx, J = tid / cnx;
-    const int dI = nt % cnx, dJ = nt / cnx;
     for (int cc = tid; cc < cn; cc += nt) {
+        const int J = local_row(Cs, cc), I = cc - J * cnx;
         float sum = 0.f;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -1082,43 +1099,40 @@ __device__ __forceinline__ void local_down(const LocalLevel Ls, const LocalLevel
             if (fi < nx && fj < ny) sum += L.t[fj * nx + fi];
         }
         C.r[cc] = sum;
-        I += dI;
-        J += dJ;
-        if (I >= cnx) { I -= cnx; ++J; }
     }
-    sync();
+    local_sync(id, nt);
 }
 
-__device__ __forceinline__ void local_up(const LocalLevel Ls, const LocalLevel Cs, float om, float alpha)
+__device__ __forceinline__ void local_up(const LocalLevel Ls, const LocalLevel Cs, float om, float alpha, int id)
 {
     const LocalView L(Ls), C(Cs);
-    const int tid = threadIdx.x, nt = blockDim.x;
-    auto sync = [] { __syncthreads(); };
-    const int nx = L.nx, ny = L.ny, n = nx * ny, cnx = C.nx;
-    auto y0 = [&](int c, int i, int j) { return L.x[c] + alpha * C.x[(j >> 1) * cnx + (i >> 1)]; };
-    int i = tid % nx, j = tid / nx;
-    const int di = nt % nx, dj = nt / nx;
-    auto step = [&] { i += di; j += dj; if (i >= nx) { i -= nx; ++j; } };
-    for (int c = tid; c < n; c += nt, step()) {   // y1 = Jacobi(y0) into t
+    const int nx = L.nx, ny = L.ny, n = nx * ny, cnx = C.nx, nt = local_threads(n), tid = threadIdx.x;
+    if (tid >= nt) return;
+    local_sync(id, nt);   // the coarse correction
+    // parents of missing neighbours: clamped into the level
+    auto y0 = [&](int c, int i, int j) {
+        return L.x[c] + alpha * C.x[(min(max(j, 0), ny - 1) >> 1) * cnx + (min(max(i, 0), nx - 1) >> 1)];
+    };
+#pragma unroll 2
+    for (int c = tid; c < n; c += nt) {   // y1 = Jacobi(y0) into t
+        const int j = local_row(Ls, c), i = c - j * nx;
         float nb = L.r[c];
-        if (i + 1 < nx) nb += L.cx[c] * y0(c + 1, i + 1, j);
-        if (i > 0) nb += L.cx[c - 1] * y0(c - 1, i - 1, j);
-        if (j + 1 < ny) nb += L.cy[c] * y0(c + nx, i, j + 1);
-        if (j > 0) nb += L.cy[c - nx] * y0(c - nx, i, j - 1);
-        L.t[c] = (1.f - om) * y0(c, i, j) + om * nb * L.id[c];
+        nb += L.cx[c] * y0(c + 1, i + 1, j);
+        nb += L.cx[c - 1] * y0(c - 1, i - 1, j);
+        nb += L.cy[c] * y0(c + nx, i, j + 1);
+        nb += L.cy[c - nx] * y0(c - nx, i, j - 1);
+        L.t[c] = __fmaf_rn(om * nb, L.id[c], __fmul_rn(1.f - om, y0(c, i, j)));
     }
-    sync();
-    i = tid % nx;
-    j = tid / nx;
-    for (int c = tid; c < n; c += nt, step()) {   // y2 = Jacobi(y1) into x
+    local_sync(id, nt);
+#pragma unroll 2
+    for (int c = tid; c < n; c += nt) {   // y2 = Jacobi(y1) into x
         float nb = L.r[c];
-        if (i + 1 < nx) nb += L.cx[c] * L.t[c + 1];
-        if (i > 0) nb += L.cx[c - 1] * L.t[c - 1];
-        if (j + 1 < ny) nb += L.cy[c] * L.t[c + nx];
-        if (j > 0) nb += L.cy[c - nx] * L.t[c - nx];
-        L.x[c] = (1.f - om) * L.t[c] + om * nb * L.id[c];
+        nb += L.cx[c] * L.t[c + 1];
+        nb += L.cx[c - 1] * L.t[c - 1];
+        nb += L.cy[c] * L.t[c + nx];
+        nb += L.cy[c - nx] * L.t[c - nx];
+        L.x[c] = __fmaf_rn(1.f - om, L.t[c], __fmul_rn(om * nb, L.id[c]));
     }
-    sync();
 }
 
 // x = A^-1 r on the direct level (n <= kDirectMax cells) from its inverse
@@ -1153,9 +1167,11 @@ __device__ __forceinline__ void local_direct(const LocalLevel Bs, int cinv)
 // S[l0].r, output S[l0].x; level ld is solved exactly.
 __device__ void vcycle_local_direct(const LocalLevel* S, int l0, int ld, int cinv, float om, float alpha)
 {
-    for (int l = l0; l < ld; ++l) local_down(S[l], S[l + 1], om);
+    for (int l = l0; l < ld; ++l) local_down(S[l], S[l + 1], om, 1 + l - l0);
+    __syncthreads();
     local_direct(S[ld], cinv);
-    for (int l = ld - 1; l >= l0; --l) local_up(S[l], S[l + 1], om, alpha);
+    for (int l = ld - 1; l >= l0; --l) local_up(S[l], S[l + 1], om, alpha, 1 + l - l0);
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(kTileBlock) mg_tile_grid_kernel(const TileArgs ta)
@@ -1174,19 +1190,19 @@ __global__ void __launch_bounds__(kTileBlock) mg_tile_grid_kernel(const TileArgs
     const int tid = threadIdx.x, nt = blockDim.x;
     const int ld = a.direct;   // levels lf..ld in CTA 0, ld solved with its inverse
     int cinv = 0;              // float offset of the inverse, after the levels
-    for (int l = lf; l <= ld; ++l) cinv += (kLocalArrays * a.lv[l].nx * a.lv[l].ny + 3) & ~3;
+    for (int l = lf; l <= ld; ++l) cinv += local_floats(a.lv[l].nx, a.lv[l].ny);
     if (b == 0) {   // the coarse levels in shared memory, with 1/d, and the inverse
         if (tid == 0) {
             int off = 0;
             for (int l = lf; l <= ld; ++l) {
-                const int n = a.lv[l].nx * a.lv[l].ny;
-                const int p = off;
-                S[l] = LocalLevel{a.lv[l].nx, a.lv[l].ny, p, p + n, p + 2 * n, p + 3 * n, p + 4 * n, p + 5 * n,
-                                  p + 6 * n};
-                off += (kLocalArrays * n + 3) & ~3;
+                const int w = a.lv[l].nx, m = w * (a.lv[l].ny + 2), p = off + w;
+                S[l] = LocalLevel{w, a.lv[l].ny, w > 1 ? (unsigned)((0x100000000ull + w - 1) / w) : 0u, p, p + m,
+                                  p + 2 * m, p + 3 * m, p + 4 * m, p + 5 * m, p + 6 * m};
+                off += local_floats(w, a.lv[l].ny);
             }
         }
         const int nd = a.lv[ld].nx * a.lv[ld].ny;
+        for (int e = tid; e < cinv; e += nt) mg_smem[e] = 0.f;   // ghost rows
         for (int e = tid; e < nd * nd; e += nt) mg_smem[cinv + e] = a.cinv[e];
         __syncthreads();
         for (int l = lf; l <= ld; ++l) {
@@ -1330,60 +1346,37 @@ __global__ void __launch_bounds__(kTileBlock) mg_tile_grid_kernel(const TileArgs
             const MgLevelDev& F = a.lv[lf - 1];
             const LocalView Lc(S[lf]);
             const int n = Lc.nx * Lc.ny;
-            // stage level lf-1's residual through the coarse level's x and t
-            // (free until its V-cycle) in chunks of whole fine-row pairs: one
-            // L2 round trip per chunk instead of one per two coarse cells
-            const int stage = S[lf].x;                  // float offset; x and t are adjacent
-            const int prows = (2 * n / F.nx) & ~1;      // fine rows per chunk
-            const bool staged = F.nx % 4 == 0 && stage % 4 == 0 && prows >= 2 &&
-                                (reinterpret_cast<size_t>(F.t) & 15) == 0;
-            if (staged) {
-                extern __shared__ __align__(16) float mg_smem_stage[];
-                float* const buf = mg_smem_stage + stage;
-                const int q4 = F.nx / 4;                // 16-byte pieces per fine row
-                for (int r0 = 0; r0 < F.ny; r0 += prows) {
-                    const int nr = min(prows, F.ny - r0);
-                    for (int k = tid; k < nr * q4; k += nt)
-                        mg_cp_async16_cg(buf + 4 * k, F.t + (size_t)r0 * F.nx + 4 * k);
-                    asm volatile("cp.async.wait_all;" ::: "memory");
-                    __syncthreads();
-                    const int J0 = r0 >> 1, J1 = min(Lc.ny, (r0 + nr + 1) >> 1);
-                    for (int k = tid; k < (J1 - J0) * Lc.nx; k += nt) {
-                        const int J = J0 + k / Lc.nx, I = k - (J - J0) * Lc.nx;
-                        float sum = 0.f;
+            // 2x2 sums of level lf-1's residual, kU coarse cells' loads in flight per
+            // thread; children in pairs where the fine rows are even (two
+            // chunks staged through shared memory took 9.8 thousand cycles on
+            // 128^2, two coarse cells at a time 7.2 on 129 x 73)
+            constexpr int kU = 4;
+            const bool even = F.nx % 2 == 0;
+            for (int c0 = 0; c0 < n; c0 += kU * nt) {
+                float2 lo[kU], hi[kU];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int gi = 2 * I + (q & 1), gj = 2 * J + (q >> 1);
-                            if (gi < F.nx && gj < F.ny) sum += buf[(gj - r0) * F.nx + gi];
+                for (int u = 0; u < kU; ++u) {
+                    const int cc = c0 + tid + u * nt;
+                    const int J = local_row(S[lf], cc), I = cc - J * Lc.nx;
+                    lo[u] = hi[u] = make_float2(0.f, 0.f);
+                    if (cc < n) {
+                        const float* f = F.t + (size_t)(2 * J) * F.nx + 2 * I;
+                        const bool up = 2 * J + 1 < F.ny, right = 2 * I + 1 < F.nx;
+                        if (even) {
+                            lo[u] = __ldcg(reinterpret_cast<const float2*>(f));
+                            if (up) hi[u] = __ldcg(reinterpret_cast<const float2*>(f + F.nx));
+                        } else {
+                            lo[u].x = __ldcg(f);
+                            if (right) lo[u].y = __ldcg(f + 1);
+                            if (up) hi[u].x = __ldcg(f + F.nx);
+                            if (up && right) hi[u].y = __ldcg(f + F.nx + 1);
                         }
-                        Lc.r[J * Lc.nx + I] = sum;
-                    }
-                    __syncthreads();
-                }
-            }
-            constexpr int kU = 2;   // coarse cells per thread whose 8 loads are in flight together
-            for (int c0 = 0; !staged && c0 < n; c0 += kU * nt) {
-                float v[kU][4];
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const int cc = c0 + tid + u * nt;
-                    const int J = cc / Lc.nx, I = cc - J * Lc.nx;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int gi = 2 * I + (q & 1), gj = 2 * J + (q >> 1);
-                        v[u][q] = cc < n && gi < F.nx && gj < F.ny ? __ldcg(F.t + gj * F.nx + gi) : 0.f;
                     }
                 }
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
                     const int cc = c0 + tid + u * nt;
-                    if (cc >= n) break;
-                    const int J = cc / Lc.nx, I = cc - J * Lc.nx;
-                    float sum = 0.f;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (2 * I + (q & 1) < F.nx && 2 * J + (q >> 1) < F.ny) sum += v[u][q];
-                    Lc.r[cc] = sum;
+                    if (cc < n) Lc.r[cc] = ((lo[u].x + lo[u].y) + hi[u].x) + hi[u].y;
                 }
             }
             __syncthreads();
@@ -2569,8 +2562,7 @@ bool tile_plan(const Plan& P, int G, TileArgs& t, size_t& smem)
     // CTA 0's coarse levels lf..ld (kLocalArrays arrays each, 16-byte
     // aligned) and the inverse of level ld's operator
     size_t local_bytes = (size_t)P.mg.nx[ld] * P.mg.ny[ld] * P.mg.nx[ld] * P.mg.ny[ld] * sizeof(float);
-    for (int l = lf; l <= ld; ++l)
-        local_bytes += (((size_t)kLocalArrays * P.mg.nx[l] * P.mg.ny[l] + 3) & ~(size_t)3) * sizeof(float);
+    for (int l = lf; l <= ld; ++l) local_bytes += (size_t)local_floats(P.mg.nx[l], P.mg.ny[l]) * sizeof(float);
     if (cap < local_bytes) return false;
     const int A = 1 << (lf - 1);
     const int gx = (P.nx + A - 1) / A, gy = (P.ny + A - 1) / A;
