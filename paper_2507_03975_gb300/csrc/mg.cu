@@ -1545,7 +1545,7 @@ __global__ void __launch_bounds__(kTileBlock) mg_tile_grid_kernel(const TileArgs
 // Bound by the latency of its ~25 dependent passes and exchanges per inner
 // iteration (16 of 152 SMs; DRAM and arithmetic idle).  Per call, before and
 // after the sends, CTA 0's small_cycle, 512 threads and the asynchronous
-// coefficient copies: 64^2 to 1e-12 213 -> 115 us, 200^2 143 -> 103 us, 256^2 with
+// coefficient copies: 64^2 to 1e-12 213 -> 120 us, 200^2 143 -> 103 us, 256^2 with
 // two inner iterations 79 -> 55 us.  The same bits.
 constexpr int kSA_D = 0, kSA_ID = 1, kSA_CX = 2, kSA_CY = 3, kSA_X = 4, kSA_T = 5, kSA_R = 6;
 constexpr int kSA_P = 7, kSA_DL = 8;   // level 0 only
@@ -1564,6 +1564,7 @@ struct SLevel {
 
 struct SArgs {
     int nl, ld, cl;
+    int lq;        // level whose rows are dealt to the CTAs: the deepest with a row for each
     SLevel lv[kMaxLevels];
     int nx, ny, N;
     const double* diag; const double* cx; const double* cy;
@@ -1591,9 +1592,9 @@ __device__ __forceinline__ float* sarr(const Strip S, int k) { return sm_f + S.o
 
 __device__ __forceinline__ void strip_rows(const SArgs& a, int l, int r, int& rs, int& re)
 {
-    const int P = a.ld + 1, nyP = a.lv[P].ny;
-    const int s0 = r * nyP / a.cl, s1 = (r + 1) * nyP / a.cl;   // below 2^25
-    const int sh = P - l;
+    const int nyQ = a.lv[a.lq].ny;
+    const int s0 = r * nyQ / a.cl, s1 = (r + 1) * nyQ / a.cl;   // below 2^25
+    const int sh = a.lq - l;
     rs = s0 << sh;
     re = min(s1 << sh, a.lv[l].ny);
 }
@@ -2200,8 +2201,8 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
             if (l == ld) {   // level P's correction: to every CTA the rows over its strip
                 if (r == 0) {
                     for (int c = C.nx + threadIdx.x; c < (C.rows + 1) * C.nx; c += blockDim.x) {
-                        const int row = c / C.nx - 1;
-                        const int q = (int)(((long long)(row + 1) * cx.size() - 1) / C.ny);   // the strip cut there
+                        const int row = (c / C.nx - 1) >> (a.lq - P);   // the row of level lq over it
+                        const int q = (int)(((long long)(row + 1) * cx.size() - 1) / a.lv[a.lq].ny);   // its CTA
                         if (q > 0) cx.send(cx.at(smem_addr(ct + c), q), ct[c], cx.xfer_bar(q));
                     }
                 } else {
@@ -2416,7 +2417,9 @@ namespace {
 // kSmallCells cells at level P.  A pass over a strip level costs an exchange
 // between the CTAs (about 1000 cycles with the pass), one inside CTA 0's
 // small_cycle 350-450 (64^2: P = 32^2 instead of 16^2).  The cut changes no
-// result: every level's arithmetic is the same in either place.
+// result: every level's arithmetic is the same in either place, and the rows
+// of a CTA, over which its dot products run, come from level `last` + 1
+// whatever the cut.
 bool strip_plan(const Plan& P, int cl, size_t smem_cap, SArgs& sa, size_t& bytes)
 {
     const MgPlan& g = P.mg;
@@ -2427,7 +2430,7 @@ bool strip_plan(const Plan& P, int cl, size_t smem_cap, SArgs& sa, size_t& bytes
     if (last < 0) return false;
     for (int ld = 0; ld <= last; ++ld) {
         if (ld < last && (long long)g.nx[ld + 1] * g.ny[ld + 1] > kSmallCells) continue;
-        const int Pl = ld + 1, nyP = g.ny[Pl];
+        const int lq = last + 1, nyQ = g.ny[lq];
         size_t off = 0;
         bool fits = true;
         for (int l = 0; l < g.nl && fits; ++l) {
@@ -2435,8 +2438,8 @@ bool strip_plan(const Plan& P, int cl, size_t smem_cap, SArgs& sa, size_t& bytes
             if (l <= ld) {
                 rows = 0;
                 for (int r = 0; r < cl; ++r) {
-                    const int s0 = (int)((long long)r * nyP / cl), s1 = (int)((long long)(r + 1) * nyP / cl);
-                    const int rs = s0 << (Pl - l), re = std::min(s1 << (Pl - l), g.ny[l]);
+                    const int s0 = (int)((long long)r * nyQ / cl), s1 = (int)((long long)(r + 1) * nyQ / cl);
+                    const int rs = s0 << (lq - l), re = std::min(s1 << (lq - l), g.ny[l]);
                     rows = std::max(rows, re - rs);
                 }
             }
@@ -2450,6 +2453,7 @@ bool strip_plan(const Plan& P, int cl, size_t smem_cap, SArgs& sa, size_t& bytes
         if (!fits) continue;
         sa.nl = g.nl;
         sa.ld = ld;
+        sa.lq = lq;
         sa.cl = cl;
         bytes = off * sizeof(float);
         return true;
