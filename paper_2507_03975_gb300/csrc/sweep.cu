@@ -473,13 +473,15 @@ struct SweepSmem {
 // after its copies in flight have landed.
 //
 // Before / after (one launch, us): FP64 64^2 S8 31 / 26, 256^2 S12 108 / 94
-// (per-ordinate source) and 189 / 150 (increment form), 200^2 S8 35 / 28 and
-// 51 / 40 (adjoint form), 1024^2 S16 919 / 887; FP32 641x470 S6 254 / 96,
+// (per-ordinate source; 88 with the south value from its slot) and 189 / 150
+// (increment form), 200^2 S8 35 / 28 (24) and 51 / 40 (36, adjoint form),
+// 1024^2 S16 919 / 887 (854); FP32 641x470 S6 254 / 96,
 // 512^2 S12 190 / 98, batch of 24 problems 158 / 128.  Bounds now: FP64 with
 // many units, the pipe (1024^2 S16: 14.2 M warp operations of 18.4 cycles on
-// 152 SMs, 0.83 ms); with few, the chain of a step (265 cycles: three FP64
-// operations and a 64-bit shuffle); FP32, instruction issue of the four warps
-// of a pair and the load warp's 34 copy instructions a chunk.
+// 152 SMs, 0.83 ms); with few, the chain of a step (253 cycles: three FP64
+// operations and the store and load of a slot; 265 with a 64-bit shuffle);
+// FP32, instruction issue of the four warps of a pair and the load warp's 34
+// copy instructions a chunk.
 template <typename T, int MODE, bool BATCH>
 __global__ void __launch_bounds__(SweepSmem<T, MODE>::THREADS, 1)
 sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
@@ -906,6 +908,10 @@ sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
                 ahead = false;
                 unsigned char* bp = buf((int)(g % NBUF));
                 T* res = reinterpret_cast<T*>(bp) + lane * RS;   // the source slots collect the results
+                // FP64, south values of steps 1.. of the chunk: lane l - 1's previous
+                // result from its slot, lane 0's from the south values
+                const volatile T* south =
+                    lane > 0 ? res - RS : reinterpret_cast<const T*>(bp + SM::off_e) + 1;
                 const int t0 = m * SEG;
                 auto steps = [&](auto wall_chunk) {
                     constexpr bool WALL = decltype(wall_chunk)::value;
@@ -922,7 +928,13 @@ sweep_kernel(const SweepArgs<T> a1, const SweepBatch<T> bt)
                         }
                         if (WALL && t0 + tt == lane) IW = wall;   // the lane's first column
                         // lane l gets lane l-1's previous result; lane 0 the south value
-                        const T Isouth = __shfl_sync(kFull, lane == 31 ? e : Iprev, (lane + 31) & 31);
+                        T Isouth;
+                        if (PRE && tt > 0) {
+                            __syncwarp();
+                            Isouth = south[tt - 1];
+                        } else {
+                            Isouth = __shfl_sync(kFull, lane == 31 ? e : Iprev, (lane + 31) & 31);
+                        }
                         T acc = fma(ai, IW, sv);
                         acc = fma(bj, Isouth, acc);
                         const T Inew = acc * rinv;
