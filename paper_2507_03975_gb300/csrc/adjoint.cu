@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kRedBlock) resid_kernel(int nx, int ny, const 
                                                           const double* __restrict__ cy, float* r0, double* partials,
                                                           double* norms, Status* status)
 {
-    __shared__ double sm[33];
+    __shared__ double sm[34];
     __shared__ int am_last;
     if (ld_volatile_int(&status->done)) return;
     const int N = nx * ny;
@@ -54,26 +54,9 @@ __global__ void __launch_bounds__(kRedBlock) resid_kernel(int nx, int ny, const 
         lrr += rv * rv;
         lbb += bv * bv;
     }
-    lrr = block_sum(lrr, sm);
-    lbb = block_sum(lbb, sm);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = lrr;
-        partials[gridDim.x + blockIdx.x] = lbb;
-        __threadfence();
-        const unsigned t = atomicAdd(&status->ticket, 1u);
-        am_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!am_last) return;
-    if (threadIdx.x < 32) {
-        __threadfence();
-        const double srr = warp_sum_array(partials, gridDim.x);
-        const double sbb = warp_sum_array(partials + gridDim.x, gridDim.x);
-        if (threadIdx.x == 0) {
-            norms[0] = srr;
-            norms[1] = sbb;
-            status->ticket = 0u;
-        }
+    if (grid_pair_sums(lrr, lbb, partials, &status->ticket, blockIdx.x, gridDim.x, sm, &am_last)) {
+        norms[0] = lrr;
+        norms[1] = lbb;
     }
 }
 
@@ -170,7 +153,7 @@ struct AdjUpdArgs {
 template <typename T>
 __global__ void __launch_bounds__(kRedBlock) adj_update_kernel(const AdjUpdArgs<T> a)
 {
-    __shared__ double sm[33];
+    __shared__ double sm[34];
     __shared__ int am_last;
     if (ld_volatile_int(&a.status->done)) return;
     double num = 0.0, den = 0.0;
@@ -186,42 +169,8 @@ __global__ void __launch_bounds__(kRedBlock) adj_update_kernel(const AdjUpdArgs<
         a.lam[c] = nw;
         a.b[c] = nw;
     }
-    num = block_sum(num, sm);
-    den = block_sum(den, sm);
-    if (threadIdx.x == 0) {
-        a.partials[blockIdx.x] = num;
-        a.partials[gridDim.x + blockIdx.x] = den;
-        __threadfence();
-        const unsigned t = atomicAdd(&a.status->ticket, 1u);
-        am_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!am_last) return;
-    if (threadIdx.x < 32) {
-        __threadfence();
-        const double sn = warp_sum_array(a.partials, gridDim.x);
-        const double sd = warp_sum_array(a.partials + gridDim.x, gridDim.x);
-        if (threadIdx.x == 0) {
-            double err;
-            if (sd > 0.0) err = sqrt(sn / sd);
-            else err = (sn == 0.0) ? 0.0 : INFINITY;
-            Status* S = a.status;
-            const int it = S->iter;
-            a.hist[it] = err;
-            S->iter = it + 1;
-            S->err = err;
-            int reason = kRunning;
-            if (!isfinite(err) || err > 1e6) reason = kDiverged;
-            else if (a.fixed_iters > 0) { if (it + 1 >= a.fixed_iters) reason = kFixedDone; }
-            else if (err < a.tol) reason = kConverged;
-            else if (it + 1 >= a.max_iter) reason = kMaxIter;
-            if (reason != kRunning) {
-                S->reason = reason;
-                S->done = 1;
-            }
-            S->ticket = 0u;
-        }
-    }
+    err_reduce_decide(num, den, a.partials, a.hist, a.status, a.tol, a.fixed_iters, a.max_iter, blockIdx.x, gridDim.x,
+                      sm, &am_last);
 }
 
 // d(HoT contribution N / (3 sigma_i S)) of owner cell i along one axis with

@@ -103,7 +103,7 @@ struct RhsArgs {
 template <bool FUSE = false>
 __device__ __forceinline__ void rhs_body(const RhsArgs& a, int bid, int nblk)
 {
-    __shared__ double sm[33];
+    __shared__ double sm[34];
     __shared__ int am_last;
     if (ld_volatile_int(&a.status->done)) return;
     const int nx = a.nx, ny = a.ny, N = nx * ny;
@@ -149,26 +149,9 @@ __device__ __forceinline__ void rhs_body(const RhsArgs& a, int bid, int nblk)
         lbb = fma(v, v, lbb);
     }
     if (!a.resid) return;   // uniform over the launch
-    lrr = block_sum(lrr, sm);
-    lbb = block_sum(lbb, sm);
-    if (threadIdx.x == 0) {
-        a.partials[bid] = lrr;
-        a.partials[nblk + bid] = lbb;
-        __threadfence();
-        const unsigned t = atomicAdd(&a.status->ticket, 1u);
-        am_last = (t == (unsigned)nblk - 1u);
-    }
-    __syncthreads();
-    if (!am_last) return;
-    if (threadIdx.x < 32) {
-        __threadfence();
-        const double srr = warp_sum_array(a.partials, nblk);
-        const double sbb = warp_sum_array(a.partials + nblk, nblk);
-        if (threadIdx.x == 0) {
-            a.norms[0] = srr;
-            a.norms[1] = sbb;
-            a.status->ticket = 0u;
-        }
+    if (grid_pair_sums(lrr, lbb, a.partials, &a.status->ticket, bid, nblk, sm, &am_last)) {
+        a.norms[0] = lrr;
+        a.norms[1] = lbb;
     }
 }
 
@@ -218,7 +201,7 @@ __device__ __forceinline__ void ordinate_row(int K, int N, int c, double sh, dou
 
 __device__ __forceinline__ void update_body(const UpdArgs& a, int bid, int nblk)
 {
-    __shared__ double sm[33];
+    __shared__ double sm[34];
     __shared__ int am_last;
     if (ld_volatile_int(&a.status->done)) return;
     double num = 0.0, den = 0.0;
@@ -244,9 +227,8 @@ __device__ __forceinline__ void update_body(const UpdArgs& a, int bid, int nblk)
             if (a.corr_f) a.corr_f[c] = (float)cc;
         }
     }
-    num = block_sum(num, sm);
-    den = block_sum(den, sm);
-    err_reduce_decide(num, den, a.partials, a.hist, a.status, a.tol, a.fixed_iters, a.max_iter, bid, nblk, &am_last);
+    err_reduce_decide(num, den, a.partials, a.hist, a.status, a.tol, a.fixed_iters, a.max_iter, bid, nblk, sm,
+                      &am_last);
 }
 
 __global__ void __launch_bounds__(kRedBlock) update_kernel(const UpdArgs a) { update_body(a, blockIdx.x, gridDim.x); }

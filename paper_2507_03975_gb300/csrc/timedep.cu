@@ -178,7 +178,7 @@ __global__ void td_coef_kernel(TdArgs a)
 // next source.
 __global__ void __launch_bounds__(kRedBlock) td_update_kernel(TdArgs a)
 {
-    __shared__ double sm[33];
+    __shared__ double sm[34];
     __shared__ int am_last;
     if (ld_volatile_int(&a.status->done)) return;
     double num = 0.0, den = 0.0;
@@ -206,10 +206,8 @@ __global__ void __launch_bounds__(kRedBlock) td_update_kernel(TdArgs a)
         a.rho_m[c] = nw;
         put_source(a, c, td_source(a, c, nw, t));
     }
-    num = block_sum(num, sm);
-    den = block_sum(den, sm);
     err_reduce_decide(num, den, a.partials, a.hist, a.status, a.tol, a.fixed_iters, a.max_iter, blockIdx.x,
-                      gridDim.x, &am_last);
+                      gridDim.x, sm, &am_last);
 }
 
 // SI: material temperature at the end of the step from the Fleck-Cummings
