@@ -380,9 +380,10 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
             }
         }
         // reflection quads (mu, eta), (-mu, eta), (mu, -eta), (-mu, -eta) of one
-        // weight: the FP64 moments then sum in fixed point (moments_fixed.cuh)
+        // weight: the FP64 moments then sum in fixed point (moments_fixed.cuh),
+        // but not in steady pseudo-time runs (moments_quads)
         std::vector<MomQuad> quads;
-        P.has_mquad = !P.fp32 && K % 4 == 0;
+        P.has_mquad = !P.fp32 && !P.pt && K % 4 == 0;
         for (int s = 0; s < K && P.has_mquad; ++s) {
             const double m = hq[s], e = hq[K + s], w = hq[2 * K + s];
             if (!(m != 0.0) || !(e != 0.0) || !(w < 2.0)) P.has_mquad = 0;
