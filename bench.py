@@ -270,10 +270,9 @@ def td_class_model(cls, prof, iters, upd, N, fp64_peak, hbm, fp64=True):
                HBM bytes at peak); bytes: read I^n once per update (8 B
                FP64, 4 B FP32) plus 64 B per cell (sigma_t, source in, six
                moments out);
-      moments: rho, F_x, F_y: over x-reflection pairs of one weight, 2 adds
-               + 3 FMA per two updates (4 FLOP per update; an add takes a
-               full FMA slot of the FP64 pipe, so the fraction is a lower
-               bound);
+      moments: rho, F_x, F_y: the intensities read once plus 48 B per cell
+               (the sums of reflection quads run in fixed point, off the
+               FP64 pipe);
       synth:   36 B per cell from HBM per call (level coefficients, r0,
                guess, x) -- bound by barriers and latency;
       hot_rhs / update: 15 / 10 doubles per cell."""
@@ -288,10 +287,7 @@ def td_class_model(cls, prof, iters, upd, N, fp64_peak, hbm, fp64=True):
         if not fp64:
             work = hbm_bytes
     elif cls == "moments":
-        work, bound, peak, unit = 4.0 * upd, ("alu" if fp64 else "hbm"), (fp64_peak if fp64 else hbm), \
-            ("GFLOP/s" if fp64 else "GB/s")
-        if not fp64:
-            work = ib * upd + 48.0 * N
+        work, bound, peak, unit = ib * upd + 48.0 * N, "hbm", hbm, "GB/s"
     elif cls == "synth":
         work, bound, peak, unit = 36.0 * N, "latency", hbm, "GB/s"
     elif cls == "hot_rhs":

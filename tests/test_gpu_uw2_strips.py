@@ -30,3 +30,18 @@ def test_two_iterations(nx, ny, order, limiter, fp32):
     o = oracle_uw2.solve(p, "si", fixed_iters=2, limiter="bj" if limiter == 0 else "none")
     err = np.abs(r["rho"].cpu().numpy() - o["rho"]).max() / np.abs(o["rho"]).max()
     assert err <= (1e-5 if fp32 else 1e-11), err
+
+
+@pytest.mark.parametrize("exponent", [-460, 460])
+def test_power_of_two_scaling_is_exact(exponent):
+    """Intensities outside the exponents for which the limiter forms its ratio
+    itself: scaling every source by a power of two scales every operation
+    exactly, so the bits are those of the unscaled run."""
+    import torch
+    from paper_2507_03975_gb300 import gsis
+    p = W.random_problem(37, 41, order=4, seed=11)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    opt = gsis.default_options(scheme=gsis.SCHEME_SI, spatial_order=2, limiter=0, fixed_iters=2, max_iter=2)
+    rho = [gsis.solve(p.dx, p.dy, p.mu, p.eta, p.w, t(p.sigma_a), t(p.sigma_s), t(p.q * s),
+                      t(p.inflow.reshape(-1) * s), opt)["rho"].cpu().numpy() / s for s in (1.0, 2.0 ** exponent)]
+    assert np.array_equal(rho[0], rho[1])
