@@ -175,42 +175,57 @@ __global__ void cell_setup_kernel(int nx, int ny, const double* __restrict__ dx,
 // Directions with the same |mu| and |eta| (the four reflections in every
 // level-symmetric set) share the value at a cell: the division, which bounds
 // this kernel, is done once, for the first of them (rrep), and stored in each
-// one's own order along the list rnext.  Two of the four orders scatter a
-// warp's store over 32 rows of the table; L2 merges them, as the neighbouring
-// steps' stores fill the same rows.  256^2 S12: 116 -> 58 us, 1024^2 S16:
-// 2.87 -> 1.34 ms.
-__global__ void recip_kernel(int nx, int ny, int nrep, int nb, const int* __restrict__ rrep,
-                             const int* __restrict__ rnext,
-                             const double* __restrict__ qmu, const double* __restrict__ qeta,
-                             const double* __restrict__ acoef, const double* __restrict__ bcoef,
-                             const double* __restrict__ sigt, const double* __restrict__ shift,
-                             double* rsw)
+// one's own order along the list rnext.  A block forms one band's values on
+// COLS columns in shared memory (columns -31 .. nx + 30: those outside the
+// mesh are zero, as are rows beyond it) and writes each order's diagonals
+// from there, a step's 32 lanes at a time: written straight from the cells,
+// two of the four orders scattered each store over 32 rows of the table.  A
+// pitch of COLS makes the diagonals conflict-free (stride COLS -+ 1, odd).
+// 256^2 S12: 116 us before the shared division, 58 before the tiles, 44 now;
+// 1024^2 S16: 2.87, 1.34, 0.84 ms (its divisions and sums take 0.55 ms of the
+// FP64 pipe); 64^2 S8 7.4 us with 16 columns (64: 14, two blocks per three SMs).
+template <int COLS>
+__global__ void __launch_bounds__(256)
+recip_kernel(int nx, int ny, int nb, const int* __restrict__ rrep, const int* __restrict__ rnext,
+             const double* __restrict__ qmu, const double* __restrict__ qeta, const double* __restrict__ acoef,
+             const double* __restrict__ bcoef, const double* __restrict__ sigt, const double* __restrict__ shift,
+             double* rsw)
 {
-    const int ns = nx + 31;
-    const size_t tot = (size_t)nrep * nb * ns * 32;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int lane = (int)(t & 31);
-        size_t u = t >> 5;
-        const int step = (int)(u % ns);
-        u /= ns;
-        const int band = (int)(u % nb);
-        const int s = rrep[u / nb];
-        const int c = step - lane, jl = band * 32 + lane;
+    __shared__ double v[32 * COLS];
+    const int ns = nx + 31, band = blockIdx.y, s = rrep[blockIdx.z];
+    const int c0 = (int)blockIdx.x * COLS - 31, c1 = min(c0 + COLS, nx + 31);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = 8;
+    int mn = rnext[s];   // the next order of the list, its signs one turn ahead
+    const bool xp = qmu[s] >= 0.0, yp = qeta[s] >= 0.0;
+#pragma unroll
+    for (int k = threadIdx.x; k < 32 * COLS; k += 256) {
+        const int c = c0 + k % COLS, jl = band * 32 + k / COLS;
+        double r = 0.0;
         if (c >= 0 && c < nx && jl < ny) {
-            const bool xp = qmu[s] >= 0.0, yp = qeta[s] >= 0.0;
             const int i = xp ? c : nx - 1 - c;
             const int j = yp ? jl : ny - 1 - jl;
             const int cell = i + nx * j;
-            const double v = 1.0 / (sigt[cell] + shift[cell] + acoef[(size_t)s * nx + i] + bcoef[(size_t)s * ny + j]);
-            for (int m = s; m >= 0; m = rnext[m]) {
-                const int mc = (qmu[m] >= 0.0) == xp ? c : nx - 1 - c;
-                const int mj = (qeta[m] >= 0.0) == yp ? jl : ny - 1 - jl;
-                rsw[(((size_t)m * nb + (mj >> 5)) * ns + mc + (mj & 31)) * 32 + (mj & 31)] = v;
-            }
-        } else {   // slots outside the mesh (the same ones in every order's own lists): zero
-            for (int m = s; m >= 0; m = rnext[m]) rsw[(((size_t)m * nb + band) * ns + step) * 32 + lane] = 0.0;
+            r = 1.0 / (sigt[cell] + shift[cell] + acoef[(size_t)s * nx + i] + bcoef[(size_t)s * ny + j]);
         }
+        v[k] = r;
+    }
+    __syncthreads();
+    const int jl = band * 32 + lane;
+    bool sx = true, sy = true;
+    for (int m = s; m >= 0;) {
+        const int mnn = mn >= 0 ? rnext[mn] : -1;
+        const double nmu = mn >= 0 ? qmu[mn] : 0.0, neta = mn >= 0 ? qeta[mn] : 0.0;
+        const int mj = sy || jl >= ny ? jl : ny - 1 - jl, ml = mj & 31;   // this row in the order of m
+        const int t0 = sx ? c0 : nx - c1;
+        double* out = rsw + ((size_t)m * nb + (mj >> 5)) * ns * 32 + ml;
+        for (int t = t0 + wid; t < t0 + (c1 - c0) + 31; t += nw) {
+            const int c = sx ? t - ml : nx - 1 - (t - ml);
+            if (t >= 0 && t < ns && c >= c0 && c < c1) out[(size_t)t * 32] = v[lane * COLS + c - c0];
+        }
+        sx = (nmu >= 0.0) == xp;
+        sy = (neta >= 0.0) == yp;
+        m = mn;
+        mn = mnn;
     }
 }
 
@@ -1526,11 +1541,17 @@ cudaError_t launch_cell_setup(const Plan& P, double cfl_p, double beta, cudaStre
         P.bface, P.gw, P.gw_f, P.sigt_d, &P.status->error);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (!P.fp32) {
-        const size_t tot = (size_t)P.nrep * P.nb * (P.nx + 31) * 32;
-        recip_kernel<<<grid_for((long long)tot, 256, P.num_sms * 16), 256, 0, st>>>(
-            P.nx, P.ny, P.nrep, P.nb, P.rrep, P.rnext, P.qmu, P.qeta, P.acoef, P.bcoef, P.sigt, P.shift,
-            const_cast<double*>(P.rsw));
+    if (!P.fp32 && P.nrep > 0) {
+        // wide tiles (fewer steps that two blocks share) where they still give
+        // every SM several blocks
+        auto tiles = [&](int cols) { return (unsigned)((P.nx + 62 + cols - 1) / cols); };
+        auto go = [&](auto kernel, int cols) {
+            kernel<<<dim3(tiles(cols), P.nb, P.nrep), 256, 0, st>>>(P.nx, P.ny, P.nb, P.rrep, P.rnext, P.qmu, P.qeta,
+                                                                    P.acoef, P.bcoef, P.sigt, P.shift,
+                                                                    const_cast<double*>(P.rsw));
+        };
+        if ((long long)tiles(64) * P.nb * P.nrep >= 4ll * P.num_sms) go(recip_kernel<64>, 64);
+        else go(recip_kernel<16>, 16);
         e = cudaGetLastError();
     }
     return e;

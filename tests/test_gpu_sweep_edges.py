@@ -32,3 +32,11 @@ def test_transport_sweep(nx, ny, order, fp32):
     tol = (4e-5 if fp32 else 1e-13) * np.abs(o["rho"]).max()
     for k, v in (("rho", o["rho"]), ("F", np.concatenate([o["Fx"], o["Fy"]])), ("bflux", o["fb"])):
         assert np.abs(r[k].cpu().numpy() - v).max() <= tol, k
+
+
+@pytest.mark.parametrize("nx,ny,order", [(1, 1, 4), (2, 33, 4), (3, 31, 4), (17, 32, 6), (18, 40, 4), (19, 64, 4),
+                                         (194, 133, 16), (195, 150, 16)])
+def test_reciprocal_tiles(nx, ny, order):
+    """Widths at which nx + 62 columns fill, just miss or just exceed the
+    reciprocal table's tiles of 16 and (the last two) 64 columns."""
+    test_transport_sweep(nx, ny, order, False)
