@@ -1671,6 +1671,11 @@ constexpr int kVirtual = 2;
 // barrier) took 1.0-1.7 thousand cycles here, and a V-cycle of the 64^2 mesh
 // has fourteen.
 //
+// A send needs a receiver whose barriers are initialised and whose arrays are
+// cleared: one cluster barrier (start) after both, before the first send.  A
+// receiver that cleared later would overwrite rows already counted as
+// arrived, and take zeros for its neighbour's values.
+//
 // Three kinds of exchange, each with its own barriers:
 //   halo       a pass's boundary rows, between neighbouring strips;
 //   sum        every CTA's partial sums, all to all;
@@ -1692,8 +1697,9 @@ class SCluster {
         n_ = (int)cl_.num_blocks();
         if (threadIdx.x < kBars) mbar_init(bars + threadIdx.x, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        cl_.sync();   // the barriers of every CTA are initialised
     }
+    // The barriers of every CTA are initialised and its arrays cleared: sends may begin.
+    __device__ void start() { cl_.sync(); }
     __device__ void sync() { cl_.sync(); }   // with global memory; also: no CTA leaves while another may store into it
     __device__ int rank() const { return rank_; }
     __device__ int size() const { return n_; }
@@ -2068,7 +2074,7 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
         float4* z4 = reinterpret_cast<float4*>(sm_f);
         for (int c = threadIdx.x; c < tot; c += blockDim.x) z4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    __syncthreads();
+    cx.start();
     // coefficients of the levels this CTA holds, and the south coupling of
     // row 0: contiguous in the level's arrays and here, so asynchronous copies
     // of 16 bytes where both sides allow it, all in flight together
