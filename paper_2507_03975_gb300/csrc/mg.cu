@@ -1575,7 +1575,7 @@ struct SArgs {
     int max_iter;
     float inner_rtol, omega, alpha;
     Status* status;
-    long long wait_cycles;   // bound of the cluster barrier's wait
+    long long wait_cycles;   // bound of an exchange's wait
 };
 
 // This CTA's part of one level: rows [rs, rs + rows); array k at float
@@ -1687,20 +1687,46 @@ constexpr int kVirtual = 2;
 // CTA has sent it something computed after its last use: a boundary cell reads
 // only the halo cell beside it, and each array's next write is at least one
 // exchange later.
+//
+// The end.  A send may only reach a CTA that has not left, and no barrier
+// waits for st.async, so a CTA leaves when it has taken everything sent to it:
+// all CTAs leave after the same sum, whose partials every one of them has
+// received.  A wait beyond the caller's bound therefore raises kErrTimeout but
+// goes on, since the CTAs of a cluster run at the same time and the bytes come;
+// the CTA marks its next partial sum, and all of them leave there.  Should a
+// wait still run out kGrace cycles later, the CTA sends nothing more and
+// leaves at once; the others follow when their waits run out, and all of them
+// give the stores in flight time to land before the last barrier (leave).
 class SCluster {
   public:
     static constexpr int kBars = 5;   // halo[2], sum[2], transfer
+    static constexpr long long kGrace = 1ll << 32;   // 2 s
+    static constexpr long long kSettle = 1ll << 21;  // 1 ms
+    static constexpr long long kTravel = 100;        // cycles: no store reaches another CTA sooner
+    // NaNs that no arithmetic makes: the partial sums of a CTA whose wait ran out
+    static constexpr unsigned kLate = 0x7fa5a5a5u;
+    static constexpr long long kLate64 = 0x7ff5a5a5a5a5a5a5ll;
     __device__ SCluster(unsigned long long* bars, long long limit, int* err)
-        : cl_(cg::this_cluster()), bars_(smem_addr(bars)), limit_(limit), err_(err), halo_(0), sum_(0), xfer_(0)
+        : cl_(cg::this_cluster()), bars_(smem_addr(bars)), limit_(limit), err_(err), halo_(0), sum_(0), xfer_(0),
+          late_(false)
     {
         rank_ = (int)cl_.block_rank();
         n_ = (int)cl_.num_blocks();
         if (threadIdx.x < kBars) mbar_init(bars + threadIdx.x, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (limit_ < kTravel && threadIdx.x < 32) raise();
     }
     // The barriers of every CTA are initialised and its arrays cleared: sends may begin.
     __device__ void start() { cl_.sync(); }
-    __device__ void sync() { cl_.sync(); }   // with global memory; also: no CTA leaves while another may store into it
+    __device__ void sync() { cl_.sync(); }   // with global memory
+    // The last call: no CTA leaves while another may store into it.
+    __device__ void leave()
+    {
+        cl_.sync();
+        if (!(ld_volatile_int(err_) & kErrTimeout)) return;   // the same in every CTA of the cluster
+        for (const long long t0 = clock64(); clock64() - t0 < kSettle;) {}
+        cl_.sync();
+    }
     __device__ int rank() const { return rank_; }
     __device__ int size() const { return n_; }
     // address in CTA q's shared memory of this CTA's shared address `a`
@@ -1733,7 +1759,7 @@ class SCluster {
     }
     // Fixed-order sums over the cluster, identical bits in every thread of
     // every CTA; also a block barrier.  slots: [2][kMaxCl][2], wsm: [64].
-    // TWO = false: only a, out[0].
+    // TWO = false: only a, out[0].  False: a wait of one of the CTAs ran out.
     template <bool TWO>
     __device__ bool sum2(const float a[kVirtual], const float b[kVirtual], float out[2], float* slots, float* ws)
     {
@@ -1761,6 +1787,7 @@ class SCluster {
                 ta += ws[w];
                 if (TWO) tb += ws[32 + w];
             }
+            if (late_) ta = __uint_as_float(kLate);
             const int q = (int)threadIdx.x;
             const unsigned dst = at(smem_addr(table + 2 * rank_), q), rb = at(bar, q);
             send(dst, ta, rb);
@@ -1770,10 +1797,12 @@ class SCluster {
         // both halves of the warp hold the table of at most 16 entries
         const int e = lane & (kMaxCl - 1);
         float s0 = e < n_ ? table[2 * e] : 0.f, s1 = TWO && e < n_ ? table[2 * e + 1] : 0.f;
+        const unsigned part = __float_as_uint(s0);
         for (int o = kMaxCl / 2; o > 0; o >>= 1) {
             s0 += __shfl_xor_sync(kFull, s0, o);
             if (TWO) s1 += __shfl_xor_sync(kFull, s1, o);
         }
+        if (isnan(s0) && __any_sync(kFull, part == kLate)) return false;
         out[0] = s0;
         out[1] = s1;
         return true;
@@ -1793,6 +1822,7 @@ class SCluster {
             double t = lane < nw ? ws[lane] : 0.0;
             for (int o = nw / 2; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
             t = __shfl_sync(kFull, t, 0);
+            if (late_) t = __longlong_as_double(kLate64);
             if (lane < n_)
                 asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
                                  at(smem_addr(table + rank_), lane)),
@@ -1801,15 +1831,18 @@ class SCluster {
         }
         if (!wait(bar, 8u * (unsigned)n_, (k >> 1) & 1u)) return false;
         double s0 = lane < n_ ? table[lane] : 0.0;
+        const long long part = __double_as_longlong(s0);
         for (int o = kMaxCl / 2; o > 0; o >>= 1) s0 += __shfl_xor_sync(kFull, s0, o);
         out = __shfl_sync(kFull, s0, 0);
-        return true;
+        return !__any_sync(kFull, part == kLate64);
     }
 
   private:
     // Phase `parity` of the barrier at shared address bar complete with `bytes`
-    // received (warp 0 polls), then a block barrier; after a wait beyond the
-    // bound kErrTimeout is raised and false returned, in every thread.
+    // received (warp 0 polls), then a block barrier; false, in every thread, if
+    // they have not come kGrace cycles after the bound.  The clock is read only
+    // if the first look, which suspends the warp for a while, finds them
+    // missing (read around every wait: 64^2 GSIS 5.93 -> 6.00 ms).
     __device__ bool wait(unsigned bar, unsigned bytes, unsigned parity)
     {
         bool ok = true;
@@ -1817,27 +1850,37 @@ class SCluster {
             if (threadIdx.x == 0)
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
             __syncwarp();
-            const long long t0 = clock64();
-            for (;;) {
-                unsigned done;
-                asm volatile("{\n\t.reg .pred p;\n\t"
-                             "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                             "selp.u32 %0, 1, 0, p;\n\t}"
-                             : "=r"(done)
-                             : "r"(bar), "r"(parity)
-                             : "memory");
-                ok = done != 0;
-                if (ok || clock64() - t0 > limit_) break;
+            ok = look(bar, parity);
+            if (!__all_sync(kFull, ok)) {
+                const long long t0 = clock64();
+                while (!(ok = look(bar, parity)) && clock64() - t0 <= limit_ + kGrace) {}
+                if (__any_sync(kFull, clock64() - t0 > limit_)) raise();
             }
-            if (!ok && threadIdx.x == 0) atomicOr(err_, kErrTimeout);
         }
         return __syncthreads_and(ok);
+    }
+    __device__ static bool look(unsigned bar, unsigned parity)
+    {
+        unsigned done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+        return done != 0;
+    }
+    __device__ void raise()   // warp 0
+    {
+        late_ = true;
+        if (threadIdx.x == 0) atomicOr(err_, kErrTimeout);
     }
     cg::cluster_group cl_;
     unsigned bars_;
     long long limit_;
     int* err_;
     unsigned halo_, sum_, xfer_;   // exchanges completed
+    bool late_;                    // warp 0: a wait took longer than the caller's bound
     int rank_, n_;
 };
 
@@ -2119,14 +2162,14 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
         if (S.prev && c < 2 * S.nx) cx.send(prev_sm + 4u * (unsigned)(S.off + k * S.cap + S.prev_rows * S.nx + c), v, pbar);
         if (S.next && c >= S.rows * S.nx) cx.send(next_sm + 4u * (unsigned)(S.off + k * S.cap + c - S.rows * S.nx), v, nbar);
     };
-    bool ok = true;
+    bool ok = true;   // false: no CTA of the cluster computes on, and this one sends no more
     // a pass that puts halo rows of strip S: `begin` before it, `end` after
     auto begin = [&] {
         pbar = cx.halo_bar(max(r - 1, 0));
         nbar = cx.halo_bar(min(r + 1, cx.size() - 1));
     };
     auto end = [&](const Strip S) {
-        ok = ok && cx.halo_wait(4u * (unsigned)S.nx * ((S.prev ? 1u : 0u) + (S.next ? 1u : 0u)));
+        ok = cx.halo_wait(4u * (unsigned)S.nx * ((S.prev ? 1u : 0u) + (S.next ? 1u : 0u)));
     };
     // One damped-Jacobi step from buffer cur into the other; its halo rows go
     // to the neighbours unless nothing reads them.
@@ -2167,7 +2210,9 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
             }
             if (strips) end(S);
             else __syncthreads();
+            if (!ok) return;
             jacobi(S, kSA_X, strips);   // X -> T
+            if (!ok) return;
             // the residual of T summed over 2x2 children
             const Strip C = St[l + 1];
             float* cr = sarr(C, kSA_R);
@@ -2194,7 +2239,8 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
             if (l < ld || !strips) __syncthreads();
             else {
                 if (r != 0) break;
-                ok = ok && cx.xfer_wait(4u * (unsigned)(C.nx * (C.rows - crows)));   // the other CTAs' rows
+                ok = cx.xfer_wait(4u * (unsigned)(C.nx * (C.rows - crows)));   // the other CTAs' rows
+                if (!ok) return;
             }
         }
         if (r == 0) small_cycle(St, wl, nl, om, alpha);
@@ -2212,7 +2258,8 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
                         if (q > 0) cx.send(cx.at(smem_addr(ct + c), q), ct[c], cx.xfer_bar(q));
                     }
                 } else {
-                    ok = ok && cx.xfer_wait(4u * (unsigned)(C.nx * ((S.rows + 1) / 2)));
+                    ok = cx.xfer_wait(4u * (unsigned)(C.nx * ((S.rows + 1) / 2)));
+                    if (!ok) return;
                 }
             }
             float* xo = sarr(S, kSA_T);
@@ -2223,7 +2270,9 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
             });
             if (strips) end(S);
             else __syncthreads();
+            if (!ok) return;
             jacobi(S, kSA_T, strips);
+            if (!ok) return;
             jacobi(S, kSA_X, false);
         }
     };
@@ -2371,7 +2420,7 @@ __device__ __forceinline__ void strip_body(const SArgs& a)
         a.status->synth_iters_total += total;
         a.status->synth_relres = bad ? kNaN : spent ? -1.0 : bb > 0.0 ? sqrt(rr / bb) : 0.0;
     }
-    cx.sync();
+    cx.leave();
 }
 
 __global__ void __launch_bounds__(kStripBlock) mg_strip_kernel(const SArgs a) { strip_body(a); }
