@@ -383,28 +383,8 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
         // weight: the FP64 moments then sum in fixed point (moments_fixed.cuh),
         // but not in steady pseudo-time runs (moments_quads)
         std::vector<MomQuad> quads;
-        P.has_mquad = !P.fp32 && !P.pt && K % 4 == 0;
-        for (int s = 0; s < K && P.has_mquad; ++s) {
-            const double m = hq[s], e = hq[K + s], w = hq[2 * K + s];
-            if (!(m != 0.0) || !(e != 0.0) || !(w < 2.0)) P.has_mquad = 0;
-            if (!(m > 0.0 && e > 0.0)) continue;
-            MomQuad q{};
-            for (int r = 0; r < 4; ++r) {
-                int t = 0;   // quads take distinct directions: a repeated direction is not a quad's
-                while (t < K && !(hq[t] == (r & 1 ? -m : m) && hq[K + t] == (r & 2 ? -e : e) && hq[2 * K + t] == w)) ++t;
-                q.s[r] = t;
-                if (t == K || (r == 0 && t != s)) P.has_mquad = 0;
-            }
-            const double cf[6] = {w, w * m, w * e, w * m * m, w * m * e, w * e * e};
-            for (int t = 0; t < 6; ++t) {
-                const unsigned long long c = (unsigned long long)std::nearbyint(std::ldexp(cf[t], 62));
-                q.c[t][0] = (unsigned)(c >> 32);
-                q.c[t][1] = (unsigned)c;
-            }
-            quads.push_back(q);
-        }
-        if (quads.size() * 4 != (size_t)K) P.has_mquad = 0;
-        if (P.has_mquad)
+        P.mquad_moments = P.fp32 || P.pt ? 0 : mom_quads(K, hq.data(), hq.data() + K, hq.data() + 2 * K, quads);
+        if (P.mquad_moments)
             CK(cudaMemcpyAsync(const_cast<MomQuad*>(P.mquad), quads.data(), quads.size() * sizeof(MomQuad),
                                cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(const_cast<double*>(P.qmu), hq.data(), hq.size() * sizeof(double),

@@ -96,7 +96,7 @@ struct Plan {
     const int* sidx;                // original k -> s
     const int* mpair;               // [K/2][2] original k of the x-reflection pairs (mu, eta), (-mu, eta), equal w
     const struct MomQuad* mquad;    // [K/4] reflection quads with fixed-point coefficients (FP64 moments)
-    int has_mquad;                  // sum over quads: the quadrature has them, no steady pseudo-time
+    int mquad_moments;              // moments summed over quads (0, 3: rho and F, 6: and P); 0 in steady pseudo-time
     const int* rrep; const int* rnext;   // [nrep] first directions of equal |mu|, |eta|; [K] the next such, or -1
     int nrep;
     int has_mpair;                  // the quadrature has such pairs: moments take the paired sums

@@ -1,7 +1,7 @@
 // Angular moments of FP64 intensities in fixed point: per cell
 //   rho = sum w I,  F = sum w Omega I,  P = sum w Omega Omega I
 // over quadrature sets closed under both axis reflections with equal weights
-// (every level-symmetric set).
+// and without very small coefficients (mom_quads; every level-symmetric set).
 //
 // Why not FP64 FMAs: GB300 issues one FP64 instruction per SM every 16
 // cycles, 64 issue slots of one sub-partition.  Five of them per pair of
@@ -19,14 +19,24 @@
 //   w eta (I1 + I2 - I3 - I4)    to F_y
 //   w mu eta (I1 - I2 - I3 + I4) to P_xy.
 // A value's 53-bit mantissa goes into a 64-bit integer d with the cell's
-// largest exponent at bit 59 (seven bits below the mantissa's own), its last
+// largest exponent at bit 60 (eight bits below the mantissa's own), its last
 // bit set (inexact values then err by less than a unit either way, without a
 // bias), so the four-term sums are exact integer additions.  Coefficients
 // are 62-bit integers c = coefficient * 2^62 (those of a moment add up to at
 // most pi), as c = 2^32 ch + 4 cl (with P, whose coefficients w mu^2 get small, all
-// 32 low bits are kept: cl there is the low word itself).  What is lost is below 2^-59 of the
-// largest intensity per term and random, against 2^-53 of the partial sum
-// per FP64 addition.  The order of the sum does not matter to integers, but
+// 32 low bits are kept: cl there is the low word itself).
+//
+// Error.  What is lost is below 2^-60 of the cell's largest intensity per
+// ordinate, times its coefficient, and random; the FP64 loop loses up to 2^-53 of
+// the partial sum per addition.  Where the largest intensity belongs to an
+// ordinate of small coefficient c, the result can be as small as c times it,
+// and the loss of the others is up to sqrt(sum c_q^2) / c times larger
+// relative to it.  mom_quads keeps that ratio below 2^8 in every moment summed
+// so: the random error is then below 1.2 2^-52, the loop's own in such a cell.
+// S16: 2^5 in rho and F, 2^7.8 in P.  Product sets with more than a few
+// polar levels, whose smallest w mu^2 are 2^-15 and less, exceed it: there the
+// loss would be 1e-13 (16 x 16), and 4e-9 in rho for a weight of 1e-9.
+// The order of the sum does not matter to integers, but
 // the scale does: where a later chunk holds a larger exponent the sums are
 // shifted down, the low bits of the high word into the next (a unit of the
 // high word is 2^-57 of the largest intensity whatever the coefficient:
@@ -36,7 +46,10 @@
 // or whose largest value is below 2^-959) take the FP64 loop.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
+#include <vector>
 
 namespace gsis {
 
@@ -47,19 +60,54 @@ struct MomQuad {
     unsigned c[6][2];
 };
 
+// Quads of the set (mu, eta, w) in `quads`, and the moments that may be summed
+// over them: 6 (rho, F, P), 3 (rho, F) or 0.  Quads take distinct directions:
+// a repeated direction is not a quad's.
+inline int mom_quads(int K, const double* mu, const double* eta, const double* w, std::vector<MomQuad>& quads)
+{
+    constexpr double kSpread = 256.0;
+    quads.clear();
+    double sum2[6] = {}, least[6] = {2.0, 2.0, 2.0, 2.0, 2.0, 2.0};
+    for (int s = 0; s < K; ++s) {
+        if (!(mu[s] != 0.0) || !(eta[s] != 0.0) || !(w[s] < 2.0)) return 0;
+        if (!(mu[s] > 0.0 && eta[s] > 0.0)) continue;
+        MomQuad q{};
+        for (int r = 0; r < 4; ++r) {
+            const double m = r & 1 ? -mu[s] : mu[s], e = r & 2 ? -eta[s] : eta[s];
+            int t = 0;
+            while (t < K && !(mu[t] == m && eta[t] == e && w[t] == w[s])) ++t;
+            if (t == K || (r == 0 && t != s)) return 0;
+            q.s[r] = t;
+        }
+        const double m = mu[s], e = eta[s], cf[6] = {w[s], w[s] * m, w[s] * e, w[s] * m * m, w[s] * m * e, w[s] * e * e};
+        for (int t = 0; t < 6; ++t) {
+            const unsigned long long c = (unsigned long long)std::nearbyint(std::ldexp(cf[t], 62));
+            q.c[t][0] = (unsigned)(c >> 32);
+            q.c[t][1] = (unsigned)c;
+            sum2[t] += cf[t] * cf[t];
+            least[t] = std::min(least[t], cf[t]);
+        }
+        quads.push_back(q);
+    }
+    if (quads.size() * 4 != (size_t)K) return 0;
+    int n = 0;
+    while (n < 6 && std::sqrt(sum2[n]) <= kSpread * least[n]) ++n;
+    return n < 3 ? 0 : n < 6 ? 3 : 6;
+}
+
 #ifdef __CUDACC__
 template <int NM>
 struct FixedMoments {
     static constexpr int kChunk = 4;   // quads whose 16 loads are in flight together
     static constexpr int kFrac = NM > 3 ? 32 : 30;   // bits of cl
-    // |dh cl| < 2^(30 + kFrac), dl cl < 2^(32 + kFrac): with 30 bits a chunk's
-    // four terms fit 64 bits, with 32 one term does
+    // |dh cl| < 2^(31 + kFrac) - 2^31, dl cl < 2^(32 + kFrac): with 30 bits a
+    // chunk's four terms and the remainder fit 64 bits, with 32 one term does
     static constexpr bool kCarryEach = kFrac == 32;
 
     long long A[NM], B2[NM];           // sum dh ch, sum dh cl
     unsigned long long B[NM];          // sum dl ch
     unsigned long long C[NM];          // sum dl cl since the last carry
-    int E;                             // the scale: biased exponent at d's bit 59
+    int E;                             // the scale: biased exponent at d's bit 60
 
     __device__ __forceinline__ void carry(int m)
     {
@@ -81,15 +129,15 @@ struct FixedMoments {
         if constexpr (kCarryEach) carry(m);
     }
 
-    // A 2^64 + B 2^32 + B2 2^(64 - kFrac), in units of 2^(E - 1144): to FP64
+    // A 2^64 + B 2^32 + B2 2^(64 - kFrac), in units of 2^(E - 1145): to FP64
     __device__ __forceinline__ double value(int m) const
     {
         const unsigned long long f = (B[m] & 0xffffffffull) + ((unsigned long long)B2[m] << (32 - kFrac));
         const long long a = A[m] + (long long)(B[m] >> 32) + (long long)(f >> 32);   // B2 < 2^kFrac: carried
         const double lo = fma((double)(unsigned)f, 0x1p-32, (double)(unsigned)a);
         const double v = fma((double)(int)(a >> 32), 0x1p32, lo);
-        // E - 1080 lies in [-1016, 966]: both factors are normal numbers
-        const int e = E - 1080, e1 = e / 2, e2 = e - e1;
+        // E - 1081 lies in [-1017, 965]: both factors are normal numbers
+        const int e = E - 1081, e1 = e / 2, e2 = e - e1;
         return v * __hiloint2double((e1 + 1023) << 20, 0) * __hiloint2double((e2 + 1023) << 20, 0);
     }
 
@@ -148,8 +196,8 @@ struct FixedMoments {
                 const unsigned h = (unsigned)(v[u] >> 32), l = (unsigned)v[u];
                 const unsigned n = (unsigned)(E - (int)((h >> 20) & 0x7ffu));   // a zero's is >= 64: shifted out
                 const unsigned mh = (h & 0xfffffu) | 0x100000u;
-                const unsigned long long m60 = ((unsigned long long)__funnelshift_l(l, mh, 7) << 32) | (l << 7);
-                v[u] = n > 63u ? 0ull : (m60 >> n) | 1ull;
+                const unsigned long long m61 = ((unsigned long long)__funnelshift_l(l, mh, 8) << 32) | (l << 8);
+                v[u] = n > 63u ? 0ull : (m61 >> n) | 1ull;
                 if (sg >> 31) v[u] = h >> 31 ? 0ull - v[u] : v[u];
             }
 #pragma unroll
@@ -177,7 +225,7 @@ struct FixedMoments {
             }
         }
         if (!ok) return false;
-        if (!any) E = 1080;
+        if (!any) E = 1081;
 #pragma unroll
         for (int m = 0; m < NM; ++m) out[m] = value(m);
         return true;

@@ -1358,23 +1358,27 @@ cudaError_t launch_sweep_batch_t(const BatchTables& bt, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// The fixed-point sums, except where the iteration amplifies the 1e-16 by
+// The fixed-point sums where the set allows them for the moments asked
+// (mom_quads), except where the iteration amplifies the 1e-16 by
 // which they differ from the loop's, so that there the sums keep their order
 // and their bits.  Second order: the limiter makes it 3e-10 within 250
-// iterations (256^2 S12 channel).  Steady pseudo-time (has_mquad is then 0):
+// iterations (256^2 S12 channel).  Steady pseudo-time (mquad_moments is then 0):
 // its runs over media of several decades stop the FP32 synthetic solve after
 // a few steps; 53x269 S14 over six decades ends 2e-9 apart, batches of such
 // meshes, whose iteration counts then differ by one, up to 2e-6.  The loop
 // takes 30.5 us there instead of 18.8 (256^2 S12), 5% of an iteration.
-const MomQuad* moments_quads(const Plan& P) { return P.has_mquad && P.order != 2 ? P.mquad : nullptr; }
+const MomQuad* moments_quads(const Plan& P, bool with_P)
+{
+    return P.mquad_moments >= (with_P ? 6 : 3) && P.order != 2 ? P.mquad : nullptr;
+}
 
 // Blocks of the cell moments: one cell per thread over reflection quads (no
 // nearly empty last turn: 1024^2 would take 3.4 turns of 8 blocks per SM),
 // else a grid-stride loop that re-uses the block's coefficient table.
 template <typename T>
-int moments_blocks(const Plan& P)
+int moments_blocks(const Plan& P, bool with_P)
 {
-    return grid_for(P.N, kRedBlock, sizeof(T) == 8 && moments_quads(P) ? INT_MAX : P.num_sms * 8);
+    return grid_for(P.N, kRedBlock, sizeof(T) == 8 && moments_quads(P, with_P) ? INT_MAX : P.num_sms * 8);
 }
 
 template <typename T>
@@ -1406,7 +1410,7 @@ cudaError_t launch_moments_t(const Plan& P, bool with_F, bool with_P, double* rh
     a.I = static_cast<const T*>(P.I);
     a.sidx = P.sidx;
     a.pairs = P.has_mpair ? P.mpair : nullptr;
-    a.quads = moments_quads(P);
+    a.quads = moments_quads(P, with_P);
     a.mu = P.omu;
     a.eta = P.oeta;
     a.w = P.ow;
@@ -1417,7 +1421,7 @@ cudaError_t launch_moments_t(const Plan& P, bool with_F, bool with_P, double* rh
     a.rho_new = gsis_correct ? P.rho_m : nullptr;
     a.done = force ? nullptr : &P.status->done;
     const size_t smem = moments_smem<T>(P.K);
-    const int grid = moments_blocks<T>(P);
+    const int grid = moments_blocks<T>(P, with_P);
     if (P.order != 2) {   // cells and boundary faces in one launch
         static_assert(kRedBlock == 256, "the boundary-flux blocks take 256 threads");
         const BfArgs<T> f = bflux_args<T>(P, fb_out, a.done);
@@ -1697,14 +1701,14 @@ int mom_batch_rec_t(const Plan& P, bool with_F, void* out)
     r.m.I = static_cast<const T*>(P.I);
     r.m.sidx = P.sidx;
     r.m.pairs = P.has_mpair ? P.mpair : nullptr;
-    r.m.quads = moments_quads(P);
+    r.m.quads = moments_quads(P, false);
     r.m.mu = P.omu; r.m.eta = P.oeta; r.m.w = P.ow;
     r.m.rho = P.rho_h;
     r.m.Fx = with_F ? P.Fx : nullptr;
     r.m.Fy = with_F ? P.Fy : nullptr;
     r.m.done = &P.status->done;
     r.f = bflux_args<T>(P, P.fb, &P.status->done);
-    r.mblocks = moments_blocks<T>(P);
+    r.mblocks = moments_blocks<T>(P, false);
     std::memcpy(out, &r, sizeof(r));
     return r.mblocks + grid_for((long long)P.nbf * 32, kRedBlock, P.num_sms * 4);
 }

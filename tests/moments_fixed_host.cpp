@@ -43,6 +43,15 @@ static void cells(const MomQuad* quads, int nq, const double* I, int n, double* 
 
 extern "C" {
 
+// The moments that may be summed in fixed point; quads: [K/4][16] words
+int set_quads(int K, const double* mu, const double* eta, const double* w, void* quads)
+{
+    std::vector<MomQuad> q;
+    const int n = mom_quads(K, mu, eta, w, q);
+    std::memcpy(quads, q.data(), std::min(q.size(), (size_t)K / 4) * sizeof(MomQuad));
+    return n;
+}
+
 // quads: [nq][16] words (4 directions, 6 coefficients in two halves); I: [K][n]; out: [n][nm]
 void fixed_cells(int nm, const void* quads, int nq, const double* I, int n, double* out, unsigned char* ok)
 {

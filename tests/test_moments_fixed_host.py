@@ -98,3 +98,75 @@ def test_level_symmetric_no_worse_than_the_loop(lib, order, kind):
         for m in range(nm):
             assert f[:, m].max() <= loop[:, m].max(), (nm, m)
             assert np.sqrt((f[:, m] ** 2).mean()) <= np.sqrt((loop[:, m] ** 2).mean()), (nm, m)
+
+
+def _product(azimuthal, polar):
+    """Gauss-Legendre levels x equally spaced angles per quadrant; the smallest w mu^2 gets very small."""
+    x, wx = np.polynomial.legendre.leggauss(2 * polar)
+    x, wx = x[polar:], wx[polar:]
+    phi = (np.arange(azimuthal) + 0.5) * np.pi / 2 / azimuthal
+    s = np.sqrt(1.0 - x * x)[:, None]
+    mu, eta = (s * np.cos(phi)).reshape(-1), (s * np.sin(phi)).reshape(-1)
+    w = np.repeat(wx, azimuthal)
+    return _all_quadrants(mu, eta, w * (np.pi / w.sum()))
+
+
+def _all_quadrants(mu, eta, w):
+    return (np.concatenate([mu, -mu, mu, -mu]), np.concatenate([eta, eta, -eta, -eta]), np.concatenate([w] * 4))
+
+
+def _small_weight(wt):
+    """S8 with one direction (and its reflections) of weight wt."""
+    mu, eta, w = W.level_symmetric_2d(8)
+    w = w.copy()
+    small = (np.abs(mu) == abs(mu[3])) & (np.abs(eta) == abs(eta[3]))
+    w[small] = wt
+    w[~small] *= (4.0 * np.pi - wt * small.sum()) / w[~small].sum()
+    return mu, eta, w
+
+
+SETS = {**{f"S{o}": W.level_symmetric_2d(o) for o in (4, 8, 16)},
+        **{f"product {a}x{p}": _product(a, p) for a, p in ((2, 1), (4, 2), (6, 3), (8, 4), (16, 16))},
+        **{f"weight {wt:g}": _small_weight(wt) for wt in (1e-2, 1e-6, 1e-9, 1e-15, 1e-20)}}
+
+
+@pytest.mark.parametrize("name", SETS)
+def test_no_set_is_worse_than_the_loop(lib, name):
+    """Of the moments that mom_quads lets through, and with the strong ordinate
+    in each direction in turn, the smallest coefficients among them."""
+    mu, eta, w = SETS[name]
+    K = len(mu)
+    table = np.zeros((K // 4, 16), np.uint32)
+    nm = lib.set_quads(K, _p(np.ascontiguousarray(mu)), _p(np.ascontiguousarray(eta)), _p(np.ascontiguousarray(w)), _p(table))
+    assert nm in (0, 3, 6)
+    assert nm == 6 if name[0] == "S" else nm == 0 if w.min() < 1e-4 else True
+    if nm == 0:
+        return
+    rng = np.random.default_rng(K)
+    for kind in ("dense", "decades", "signed", "rising", "beam"):
+        I = _intensities(kind, _quads(mu, eta), rng)
+        if kind == "beam":   # all directions alike
+            I[:] = rng.uniform(0.5, 1.0, I.shape) * 10.0 ** rng.uniform(-12.0, -2.0, (1, CELLS))
+            I[np.arange(CELLS) % K, np.arange(CELLS)] = rng.uniform(1.0, 2.0, CELLS)
+        fixed, loop = _errors(lib, mu, eta, w, table, I)
+        for n in (1, 3, 6)[:{3: 2, 6: 3}[nm]]:
+            for m in range(n):
+                assert fixed[n][:, m].max() <= loop[:, m].max(), (kind, n, m)
+                assert np.sqrt((fixed[n][:, m] ** 2).mean()) <= np.sqrt((loop[:, m] ** 2).mean()), (kind, n, m)
+
+
+@pytest.mark.parametrize("value", [2.0 - 2.0 ** -52, -(2.0 - 2.0 ** -52)])
+@pytest.mark.parametrize("name", SETS)
+def test_largest_sums_fit(lib, name, value):
+    """All mantissas full: the sums reach their largest magnitudes."""
+    mu, eta, w = SETS[name]
+    K = len(mu)
+    table = np.zeros((K // 4, 16), np.uint32)
+    nm = lib.set_quads(K, _p(np.ascontiguousarray(mu)), _p(np.ascontiguousarray(eta)), _p(np.ascontiguousarray(w)), _p(table))
+    for n in (3, 6):
+        if n > nm:
+            continue
+        I, out, ok = np.full((K, 1), value), np.empty((1, n)), np.zeros(1, np.uint8)
+        lib.fixed_cells(n, _p(table), K // 4, _p(I), 1, _p(out), _p(ok))
+        ref = np.array([(w * f).sum() * value for f in (1.0, 0 * mu, 0 * eta, mu * mu, 0 * mu, eta * eta)])[:n]
+        assert ok[0] and np.abs(out[0] - ref).max() < 1e-14 * abs(ref[0])
