@@ -31,6 +31,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "divide.cuh"
 #include "gsis_internal.cuh"
 #include "moments_fixed.cuh"
 
@@ -309,21 +310,6 @@ struct SweepBatch {
     int* err;                    // the launch's own error bits (a wait outside any unit)
     long long wait_cycles;
 };
-
-// 1/d of an FP32 diagonal in [2^-100, 2^100], correctly rounded: one Newton
-// step r + r (1 - d r) with the residual exact by FMA, from an approximation
-// within 1 ulp (Markstein 1990, "Computation of elementary functions on the
-// IBM RISC System/6000"; compared with __frcp_rn for every float of the
-// range: equal).  Six instructions that overlap from cell to cell;
-// __frcp_rn with its range checks took 136 cycles a cell, one after the
-// other, and set the pace of the FP32 sweep (2179 cycles per 16-step chunk).
-constexpr unsigned kRcpLo = (127u - 100u) << 23, kRcpHi = (127u + 100u) << 23;
-__device__ __forceinline__ float rcp_newton(float d)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return __fmaf_rn(r, __fmaf_rn(-d, r, 1.0f), r);
-}
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem)

@@ -19,6 +19,7 @@
 // global memory.
 #include <cuda_runtime.h>
 
+#include "divide.cuh"
 #include "gsis_internal.cuh"
 
 namespace gsis {
@@ -87,29 +88,6 @@ __device__ __forceinline__ void limited_gradient(const Uw2Args<T>& a, const T* I
                           a.limiter, gx, gy);
 }
 
-// a / d for 0 <= a < d, the bits of the division: reciprocal from the FP32
-// approximation of d's leading 24 bits (integer instructions), one third-order
-// Newton step, and the quotient corrected by its exact residual (Markstein
-// 1990; compared with the division on 5e8 pairs: equal).  Six FP64 operations
-// and no branch taken; the division is 140 cycles of the pipe and a call that
-// keeps the other rows' work from overlapping (256^2 S12: 554 -> 482 us).
-// Exponents outside the checked range take the division.
-__device__ __forceinline__ double ratio(double a, double d)
-{
-    const unsigned dh = (unsigned)__double2hiint(d), ah = (unsigned)__double2hiint(a);
-    const unsigned ed = dh >> 20, ea = ah >> 20;
-    if (ed - 600u > 800u || (ea - 400u > 1000u && __double_as_longlong(a) != 0)) return a / d;
-    const float m = __uint_as_float(0x3f800000u | (__funnelshift_l((unsigned)__double2loint(d), dh, 3) & 0x7fffffu));
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));
-    const unsigned rb = __float_as_uint(r);
-    const double y0 = __hiloint2double((int)((rb >> 3) + ((1023u - 127u + 1023u - ed) << 20)), (int)(rb << 29));
-    const double e = fma(-d, y0, 1.0);
-    const double y = fma(y0, fma(e, e, e), y0);
-    const double q = a * y;
-    return fma(fma(-q, d, a), y, q);
-}
-
 // The Barth-Jespersen factor from the differences to the neighbours, east,
 // west (negated), ahead, behind (negated; 0 where there is none) and the face
 // changes hx/2 G_x, hy/2 G_y: false where the limiter does not act.  Rounding is
@@ -138,17 +116,6 @@ __device__ __forceinline__ bool limit(float dE, float dWn, float dA, float dBn, 
     psi = room / dm;
     return true;
 }
-
-// x / h with y = 1/h correctly rounded: the quotient x y corrected by its exact
-// residual is the correctly rounded one (Markstein 1990, "Computation of
-// elementary functions on the IBM RISC System/6000"), so the bits of x / h, in
-// three FP64 operations.
-__device__ __forceinline__ double div_by(double x, double h, double y)
-{
-    const double q = x * y;
-    return fma(fma(-q, h, x), y, q);
-}
-__device__ __forceinline__ float div_by(float x, float h, float) { return x / h; }
 
 // Residual, one warp per ordinate, 29 columns and kUwRows rows.  The FP64
 // pipe bounds it, so every quantity that two cells share is formed once:
