@@ -45,6 +45,26 @@ __global__ void check_ratio(u64* bad, int per, int mode, int range)
     }
 }
 
+// The same modes; 1: the mesh width's mantissa next to a power of two.  Beyond
+// the exponents that div_by states, the last place may differ.
+__global__ void check_div_by(u64* bad, int per, int mode, int range)
+{
+    const u64 id = blockIdx.x * (u64)blockDim.x + threadIdx.x;
+    for (int i = 0; i < per; ++i) {
+        const u64 r = mix(id * per + i), t = mix(r ^ 0x7654321);
+        const u64 eh = range ? 523 + (r >> 53) % 1000 : 990 + (r >> 54) % 70, ex = range ? t >> 53 : eh - (t >> 56) % 60;
+        const u64 mh = mantissa(r, mode == 1), mx = mode == 2 ? mh + (t & 127) - 64 : t;
+        const double h = make(eh, mh), y = 1.0 / h;
+        double x = i % 97 == 0 ? 0.0 : make(ex < 2047 ? ex : 2046, mx);
+        if (t >> 20 & 1) x = -x;
+        const double q = x / h, ax = fabs(x), aq = fabs(q);
+        if (isinf(q)) continue;
+        const bool inside = x == 0.0 || (ax >= 0x1p-960 && ax <= 0x1p960 && aq >= 0x1p-1000 && aq <= 0x1p1000);
+        const long long off = __double_as_longlong(div_by(x, h, y)) - __double_as_longlong(q);
+        if (off < (inside ? 0 : -1) || off > (inside ? 0 : 1)) atomicAdd(bad, 1ull);
+    }
+}
+
 int main()
 {
     u64* bad;
@@ -67,6 +87,8 @@ int main()
         for (int range = 0; range < 2; ++range) {
             check_ratio<<<B, T>>>(bad, N, mode, range);
             if (!report("ratio")) return 1;
+            check_div_by<<<B, T>>>(bad, N, mode, range);
+            if (!report("div_by")) return 1;
         }
     return 0;
 }

@@ -1,7 +1,7 @@
 """The reciprocals and quotients of csrc/divide.cuh have the bits of the
 device's division: every float of rcp_newton's range, and for the FP64
 quotients random pairs, mantissas where rounding is hardest, and all
-exponents (beyond the ranges in which they work without it, too)."""
+exponents (where div_by states no equality: the last place)."""
 import subprocess
 from pathlib import Path
 
@@ -20,4 +20,4 @@ def test_same_bits_as_the_division(tmp_path):
     out = subprocess.run([exe], capture_output=True, text=True, timeout=120)
     assert out.returncode == 0, out.stdout + out.stderr
     lines = out.stdout.split("\n")[:-1]
-    assert len(lines) >= 7 and all(line.split()[-1] == "0" for line in lines), out.stdout
+    assert len(lines) >= 13 and all(line.split()[-1] == "0" for line in lines), out.stdout
