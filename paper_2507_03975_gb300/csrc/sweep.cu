@@ -1294,22 +1294,35 @@ SweepArgs<T> sweep_args(const Plan& P)
     return a;
 }
 
-// One problem's sweep: a cooperative launch, which guarantees the whole grid
+// One problem's sweep.  A cooperative launch guarantees the whole grid
 // resident, so the units are placed without a check-in and the warps leave
-// without counting (64^2 S8 source iteration 46.5 -> 44.5 us per iteration);
-// where it does not fit the SMs that the context may use, the plain launch
-// with its check-in.
+// without counting: 2 us less, of 38 to 130 per iteration.  But it starts only
+// when its whole grid fits, so that the sweeps of several streams take turns
+// where plain launches share the SMs.  Source iteration on meshes 64 cells
+// wide, us an iteration with 1 / 2 / 4 / 8 streams, cooperative | plain | the
+// sweep before the roles of its warps were split (plain):
+//   24 CTAs  44 / 46 /  52 /  63 | 46 / 48 /  53 /  65 |  59 /  63 /  78 / 118
+//   60       65 / 67 /  75 / 137 | 66 / 69 /  77 / 113 |  86 /  91 / 110 / 168
+//   72       71 / 73 /  95 / 187 | 73 / 75 /  90 / 133 |  95 /  99 / 125 / 185
+//   84       77 / 79 / 120 / 238 | 79 / 82 / 100 / 145 | 103 / 108 / 136 / 205
+//   96       85 / 88 / 156       | 86 / 89 / 112 / 163 | 113 / 120 / 150 / 222
+// (152 CTAs, 128^2 S8: 69 / 100 / 196 | 71 / 90 / 116).  So cooperative where two
+// such launches fit at once: there no number of streams is slower than with
+// that form.  Beyond, and where the grid does not fit the SMs that the context
+// may use, plain with its check-in.
 template <typename T, int MODE>
-cudaError_t launch_sweep_args(SweepArgs<T> a, int grid, cudaStream_t st)
+cudaError_t launch_sweep_args(SweepArgs<T> a, int grid, int num_sms, cudaStream_t st)
 {
     using SM = SweepSmem<T, MODE>;
     SweepBatch<T> none{};
-    a.resident = 1;
-    void* args[] = {&a, &none};
-    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)sweep_kernel<T, MODE, false>, dim3(grid),
-                                                      dim3(SM::THREADS), args, SM::bytes, st);
-    if (e != cudaErrorCooperativeLaunchTooLarge) return e;
-    cudaGetLastError();
+    if (2 * grid <= num_sms) {
+        a.resident = 1;
+        void* args[] = {&a, &none};
+        const cudaError_t e = cudaLaunchCooperativeKernel((const void*)sweep_kernel<T, MODE, false>, dim3(grid),
+                                                          dim3(SM::THREADS), args, SM::bytes, st);
+        if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+        cudaGetLastError();
+    }
     a.resident = 0;
     sweep_kernel<T, MODE, false><<<grid, SM::THREADS, SM::bytes, st>>>(a, none);
     return cudaGetLastError();
@@ -1319,7 +1332,7 @@ template <typename T, int MODE>
 cudaError_t launch_sweep_t(Plan& P, cudaStream_t st)
 {
     const SweepArgs<T> a = sweep_args<T, MODE>(P);
-    return launch_sweep_args<T, MODE>(a, P.sweep_grid, st);
+    return launch_sweep_args<T, MODE>(a, P.sweep_grid, P.num_sms, st);
 }
 
 template <typename T, int MODE>
@@ -1586,7 +1599,7 @@ cudaError_t launch_sweep(Plan& P, cudaStream_t st)
         SweepArgs<double> a = sweep_args<double, kSrcPlain>(P);
         a.src = P.X;
         a.src_stride = P.N;
-        return launch_sweep_args<double, kSrcPlain>(a, P.sweep_grid, st);
+        return launch_sweep_args<double, kSrcPlain>(a, P.sweep_grid, P.num_sms, st);
     }
     if (P.fp32 && P.pt && P.X_f) {
         // FP32 time step with its source combined per ordinate (X = src +
@@ -1596,7 +1609,7 @@ cudaError_t launch_sweep(Plan& P, cudaStream_t st)
         a.src = P.X_f;
         a.src_stride = P.N;
         a.sigt = P.sigt_d;
-        return launch_sweep_args<float, kSrcPlain>(a, P.sweep_grid, st);
+        return launch_sweep_args<float, kSrcPlain>(a, P.sweep_grid, P.num_sms, st);
     }
     if (P.fp32) {
         return P.pt ? launch_sweep_t<float, kSrcPseudoTime>(P, st)
@@ -1623,7 +1636,7 @@ cudaError_t launch_sweep_pt_into_t(Plan& P, const void* src, const void* iold, v
     a.iold = static_cast<const T*>(iold);
     a.I = static_cast<T*>(out);
     a.inflow = nullptr;
-    return launch_sweep_args<T, kSrcPseudoTime>(a, P.sweep_grid, st);
+    return launch_sweep_args<T, kSrcPseudoTime>(a, P.sweep_grid, P.num_sms, st);
 }
 
 cudaError_t launch_sweep_pt_into(Plan& P, const void* src, const void* iold, void* out, cudaStream_t st)
