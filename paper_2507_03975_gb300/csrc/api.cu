@@ -19,6 +19,7 @@
 #include "gsis_internal.cuh"
 #include "host.h"
 #include "moments_fixed.cuh"
+#include "reflections.h"
 
 using namespace gsis;
 
@@ -369,16 +370,7 @@ int prepare(Plan& P, const gsis_mesh* mesh, const gsis_quadrature* quad, const g
             }
         }
         // directions of equal |mu|, |eta| (they share 1/d at a cell): first ones and chains
-        P.nrep = 0;
-        for (int s = 0; s < K; ++s) {
-            int f = 0;
-            while (std::fabs(hq[f]) != std::fabs(hq[s]) || std::fabs(hq[K + f]) != std::fabs(hq[K + s])) ++f;
-            if (f == s) hi[3 * K + P.nrep++] = s;
-            else {
-                while (hi[4 * K + f] >= 0) f = hi[4 * K + f];
-                hi[4 * K + f] = s;
-            }
-        }
+        P.nrep = reflection_chains(K, hq.data(), hq.data() + K, hi.data() + 3 * (size_t)K, hi.data() + 4 * (size_t)K);
         // reflection quads (mu, eta), (-mu, eta), (mu, -eta), (-mu, -eta) of one
         // weight: the FP64 moments then sum in fixed point (moments_fixed.cuh),
         // but not in steady pseudo-time runs (moments_quads)

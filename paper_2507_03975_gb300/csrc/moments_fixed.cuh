@@ -51,6 +51,8 @@
 #include <cstdint>
 #include <vector>
 
+#include "reflections.h"
+
 namespace gsis {
 
 // One quad of the set: the four sorted directions and, per moment (rho, F_x,
@@ -67,19 +69,27 @@ inline int mom_quads(int K, const double* mu, const double* eta, const double* w
 {
     constexpr double kSpread = 256.0;
     quads.clear();
-    double sum2[6] = {}, least[6] = {2.0, 2.0, 2.0, 2.0, 2.0, 2.0};
-    for (int s = 0; s < K; ++s) {
+    for (int s = 0; s < K; ++s)
         if (!(mu[s] != 0.0) || !(eta[s] != 0.0) || !(w[s] < 2.0)) return 0;
-        if (!(mu[s] > 0.0 && eta[s] > 0.0)) continue;
+    if (K % 4 != 0) return 0;
+    const std::vector<int> at = by_magnitude(K, mu, eta, w);
+    double sum2[6] = {}, least[6] = {2.0, 2.0, 2.0, 2.0, 2.0, 2.0};
+    for (int i = 0; i < K; i += 4) {
         MomQuad q{};
+        unsigned signs = 0;
+        const int a = at[i];
+        auto alike = [&](int b) {
+            return std::fabs(mu[b]) == std::fabs(mu[a]) && std::fabs(eta[b]) == std::fabs(eta[a]) && w[b] == w[a];
+        };
         for (int r = 0; r < 4; ++r) {
-            const double m = r & 1 ? -mu[s] : mu[s], e = r & 2 ? -eta[s] : eta[s];
-            int t = 0;
-            while (t < K && !(mu[t] == m && eta[t] == e && w[t] == w[s])) ++t;
-            if (t == K || (r == 0 && t != s)) return 0;
-            q.s[r] = t;
+            const int t = at[i + r], sign = (mu[t] < 0.0 ? 1 : 0) + (eta[t] < 0.0 ? 2 : 0);
+            if (!alike(t)) return 0;
+            signs |= 1u << sign;
+            q.s[sign] = t;
         }
-        const double m = mu[s], e = eta[s], cf[6] = {w[s], w[s] * m, w[s] * e, w[s] * m * m, w[s] * m * e, w[s] * e * e};
+        if (signs != 15u || (i + 4 < K && alike(at[i + 4]))) return 0;
+        const double m = std::fabs(mu[a]), e = std::fabs(eta[a]);
+        const double cf[6] = {w[a], w[a] * m, w[a] * e, w[a] * m * m, w[a] * m * e, w[a] * e * e};
         for (int t = 0; t < 6; ++t) {
             const unsigned long long c = (unsigned long long)std::nearbyint(std::ldexp(cf[t], 62));
             q.c[t][0] = (unsigned)(c >> 32);
@@ -89,7 +99,7 @@ inline int mom_quads(int K, const double* mu, const double* eta, const double* w
         }
         quads.push_back(q);
     }
-    if (quads.size() * 4 != (size_t)K) return 0;
+    std::sort(quads.begin(), quads.end(), [](const MomQuad& a, const MomQuad& b) { return a.s[0] < b.s[0]; });
     int n = 0;
     while (n < 6 && std::sqrt(sum2[n]) <= kSpread * least[n]) ++n;
     return n < 3 ? 0 : n < 6 ? 3 : 6;

@@ -52,6 +52,12 @@ int set_quads(int K, const double* mu, const double* eta, const double* w, void*
     return n;
 }
 
+// First directions of equal |mu|, |eta| and chains
+int chains(int K, const double* mu, const double* eta, int* rep, int* next)
+{
+    return reflection_chains(K, mu, eta, rep, next);
+}
+
 // quads: [nq][16] words (4 directions, 6 coefficients in two halves); I: [K][n]; out: [n][nm]
 void fixed_cells(int nm, const void* quads, int nq, const double* I, int n, double* out, unsigned char* ok)
 {
