@@ -267,9 +267,8 @@ constexpr int kSrcPlain = 0, kSrcPseudoTime = 1, kSrcAdjoint = 2, kSrcDelta = 3;
 // pseudo-time, adjoint and increment forms read two per-cell/per-ordinate
 // arrays more, the plain form none.  (A time-step form that read I^n and
 // the per-cell source, one window more, with 1/(c dt) as a constant, was
-// measured slower: 1024^2 S16 sweep 1.09 -> 1.92 ms against the 0.40 ms of
-// the per-ordinate source pass it saved; the sweep is bound by its copy
-// pipeline.)
+// measured when a pair had two warps, one for the copies: 1024^2 S16 sweep
+// 1.09 -> 1.92 ms against the 0.40 ms of the per-ordinate source pass it saved.)
 __host__ __device__ constexpr int sweep_xw(int mode) { return mode == kSrcPlain ? 0 : 2; }
 
 template <typename T>
@@ -437,8 +436,8 @@ struct SweepSmem {
 // One persistent CTA per SM runs PAIRS "pairs" of a compute warp and its two
 // or three helpers; a pair's load warp chooses the units (direction s, band),
 // u = band * K + s, and hands each on in the headers of its chunk buffers.
-// When the whole grid is resident (every CTA checks in within a few
-// microseconds) the units are placed statically: pair p of CTA c takes
+// When the whole grid is resident (a cooperative launch, or every CTA checks in
+// within a few microseconds) the units are placed statically: pair p of CTA c takes
 // u = p G + c + i PAIRS G, so each SM's first units come from different
 // bands and run at different times; every unit is owned by a running pair and
 // waits only on u - K.  Otherwise (part of the grid held back by other work

@@ -1,6 +1,6 @@
-"""The second-order residual kernel at the edges of its strips (29 columns, 32
-rows) and of its warps of ordinates (8 per block), with and without the
-limiter, on a non-uniform mesh with inflow.
+"""The second-order residual kernel at the edges of its strips' width (29
+columns) and over several strips of 16 rows, with and without the limiter, on
+a non-uniform mesh with inflow.
 
 Tolerance: the kernel's operations are the oracle's up to the order of a few
 roundings; two iterations of the scheme amplify 1e-16 by less than 1e4 on
