@@ -163,14 +163,14 @@ def _clock_summary(proc, f, uuid, index):
 
 
 # DRAM bytes per launch from ncu captures (dram__bytes_read.sum +
-# dram__bytes_write.sum, one capture each, summarised in profiles/), valid
-# while the sources that define the sweep launch (kernel, arguments, grid,
-# workspace layout) are the captured ones.
+# dram__bytes_write.sum, one capture each), valid while the sources that define
+# the sweep launch (kernel, arguments, grid, workspace layout) are the captured
+# ones.
 SWEEP_SOURCES = ("sweep.cu", "gsis_internal.cuh", "host.h", "api.cu", "timedep.cu", "batch.cu")
 SWEEP_TRAFFIC = {   # {workload: (sources digest, bytes per launch)}
-    "timedep_fp64": ("015e39fc02e2b184", 3_766_858_240),   # profiles/sweep_kernel_traffic.md
-    "channel": ("015e39fc02e2b184", 109_599_232),          # profiles/sweep_kernel_traffic.md
-    "batch": ("015e39fc02e2b184", 982_848_256),            # profiles/sweep_kernel_traffic.md
+    "timedep_fp64": ("bca9b92b31075d47", 3_764_646_656),
+    "channel": ("bca9b92b31075d47", 109_574_912),
+    "batch": ("bca9b92b31075d47", 982_704_896),
 }
 
 
